@@ -891,7 +891,7 @@ def large_leg(talekpir, synth, torch, stream, args, hbm_peak) -> dict:
     return {"n": n, "d": d, "msg_bytes": z, "B": B, "table_bytes": tb,
             "batched_ms": bms, "batched_reads_per_s": B / (bms * 1e-3),
             "batched_lop3_equivalent_tops": ops / (bms * 1e-3) / 1e12,
-            "batched_kernel": "gf2_mma_kernel (automatic choice at B = 1024)",
+            "batched_kernel": "tensor-core kernel (automatic choice at B = 1024)",
             "batched_tensor_tflops": gf2_mma_flops(n, d * z, B) / (bms * 1e-3) / 1e12,
             "m4rm_kernel_ms": mms, "m4rm_kernel_reads_per_s": B / (mms * 1e-3),
             "lop3_kernel_ms": lms, "lop3_kernel_reads_per_s": B / (lms * 1e-3),

@@ -217,8 +217,10 @@ tpir_status tpir_xor_combine(const void *const *d_srcs, uint32_t count, uint64_t
                              void *d_dst, void *stream);
 
 /* Force a kernel choice for tests and benchmarks: 0 = automatic (plain for
- * B <= 4, tensor-core for B >= 48 on rows of >= 256 bytes, register-tiled
- * batched otherwise), 1 = plain streaming kernel (B <= 4 per launch,
+ * B <= 4, tensor-core for B >= 48 on rows of >= 256 bytes, and from the
+ * second such batch of a table for narrower rows and for the smaller batches
+ * it is faster at; register-tiled batched otherwise, and where there is no room
+ * for the tensor-core kernel's copy of the table), 1 = plain streaming kernel (B <= 4 per launch,
  * larger B is split into launches; TMA-staged where the row width allows),
  * 2 = batched register-tiled kernel, 3 = plain kernel with register
  * streaming only (the path used for row widths the TMA-staged one skips),
@@ -226,10 +228,10 @@ tpir_status tpir_xor_combine(const void *const *d_srcs, uint32_t count, uint64_t
  * shared memory, one lookup per request and group), 5 = batched tensor-core
  * kernel (the GF(2) product as an exact integer product of 0/1 matrices on
  * tcgen05: packed 4-bit e2m1 operands with unit block scales, fp32
- * accumulators, reduced mod 2; batches of more than 128 requests run on
- * pairs of SMs sharing each M = 256 MMA, cta_group::2, unless a tuning plan
- * chose single CTAs; a device that cannot hold the pairs' clusters takes
- * single CTAs).  The tensor-core kernel reads a
+ * accumulators, reduced mod 2; the table operand is held in tensor memory, or,
+ * for batches of more than 128 requests where that is estimated or was tuned
+ * to be faster, both are in shared memory and pairs of SMs share each M = 256
+ * MMA, cta_group::2).  The tensor-core kernel reads a
  * bit-transposed copy of the table (each column's bits over 64 buckets in
  * one word; as large as the table), allocated and built by the first read
  * that uses it and then kept equal to the table by every write and load. */
@@ -240,11 +242,9 @@ tpir_status tpir_db_set_kernel(tpir_db *db, int kernel);
  *   - every admissible tile shape of the register-tiled kernel (lanes along
  *     the row, warps along requests / row / buckets, i.e. the batch tile
  *     width and the row tile width, and the rows per pipeline stage);
- *   - the tensor-core kernel's schedules (equal spans of stages per CTA, or
- *     items of whole k-chunks of 4096 .. 32768 buckets or the planned size;
- *     request words staged by TMA or loaded by the expander threads; above
- *     128 requests items on CTA pairs and on single CTAs) when rows are 256
- *     bytes or wider;
+ *   - the tensor-core kernel's schedules (the table operand in tensor memory;
+ *     above 128 requests also items on CTA pairs; each with k-chunks of the
+ *     planned size and of 2048 .. 32768 buckets);
  *   - the Four-Russians kernel (B >= 32, rows of 256 bytes or more) and the
  *     plain kernel (B <= 16);
  * and keeps (a) the fastest tile shape for every later launch of the
@@ -262,9 +262,9 @@ typedef struct {
     double us_per_launch;      /* of the chosen register-tiled shape */
     double lop3_tops;          /* B*n*row_words / time */
     uint32_t kernel;           /* fastest kernel (as in tpir_db_set_kernel) */
-    uint32_t tensor_mode;      /* its tensor-core schedule: 1 spans, 2 items (on CTA pairs above
-                                  128 requests), 3 items on single CTAs */
-    uint32_t tensor_kc_rows;   /* items: k-chunk buckets (0: planned size) */
+    uint32_t tensor_mode;      /* its tensor-core schedule: 1 table operand in tensor memory, 2
+                                  items on CTA pairs (above 128 requests) */
+    uint32_t tensor_kc_rows;   /* k-chunk buckets (0: planned size) */
     uint32_t tensor_loads;     /* 1: request words loaded by threads, not TMA */
     uint32_t tensor_candidates;
     double us_lop3, us_tensor, us_m4rm, us_plain;  /* best of each kernel (0: not timed) */
@@ -279,10 +279,9 @@ tpir_status tpir_tune_clear(void);
 /* Many tables in ONE persistent launch per kernel kind (the uneven-batching
  * workload): job i reads B_i rows of d_req_bits_i against db_i into d_out_i.
  * Tables may differ in n, d and msg_bytes.  Jobs of >= 48 requests on rows of
- * >= 256 bytes go to the tensor-core kernel: those of more than 128 requests
- * on tables of >= 8192 buckets share one CTA-pair launch, the rest one
- * single-CTA launch (each per request-staging mode), the others one
- * launch of the register-tiled kernel (a db forced to kernel 4 sends its jobs
+ * >= 256 bytes, and smaller ones the tensor-core kernel is faster at on tables
+ * that have its copy, share one launch of the tensor-core kernel (per 64 jobs),
+ * the others one launch of the register-tiled kernel (a db forced to kernel 4 sends its jobs
  * to the Four-Russians kernel instead: one launch for jobs of up to 256
  * requests, one for larger ones; forced to 2, to the register-tiled one).  A
  * job with d_seeds (B x 32 bytes, 16-byte aligned) is masked as in

@@ -142,12 +142,26 @@ int auto_kernel(const tpir_db* db, uint32_t B) {
   if (db->forced_kernel) return db->forced_kernel;
   KernelPlan kp;
   if (kernel_plan_lookup(db->Wd, B, db->n, &kp)) return kp.kernel;  // measured winner
-  // plain stream for a few requests; the tensor-core kernel once its
-  // 128-request M-tiles are well filled (measured crossover with the
-  // register-tiled kernel on GB300); the register-tiled kernel in between
+  // plain stream for a few requests; the tensor-core kernel for large batches
+  // on wide rows, and for the others it is faster at (tensor_mid) once the
+  // table has its transposed copy, or had one such batch before: the first
+  // runs on the register-tiled kernel, so that a table read once does not pay
+  // for the copy
   if (B <= kPlainMaxB) return 1;
-  if (B >= kTensorMinB && db->Wd >= 64) return 5;
-  return 2;
+  if (tensor_mid(db, B)) return !db->tt_denied && (db->tt_valid || db->mid_reads) ? 5 : 2;
+  return B >= kTensorMinB && db->Wd >= kTensorMinWd && !db->tt_denied ? 5 : 2;
+}
+
+// Batches other than the large ones on wide rows that the tensor-core kernel
+// reads faster than the register-tiled one (us, tensor / register-tiled: 8 192
+// x 4 KiB 13 / 31 at 8 requests, 17 / 25 at 32; 32 768 x 4 KiB 38 / 32, 38 / 39,
+// 38 / 44, 39 / 70 at 5, 8, 16, 32; 131 072 x 4 KiB 127 / 98, 127 / 144 at 8, 16;
+// 200 003 x 256 bytes 18 / 68 at 5; 200 003 x 128 bytes 14 / 93 at 64): up to 8
+// requests the register-tiled kernel streams large tables of wide rows from
+// HBM at a higher rate.
+bool tensor_mid(const tpir_db* db, uint32_t B) {
+  if (B <= kPlainMaxB || (B >= kTensorMinB && db->Wd >= kTensorMinWd)) return false;
+  return B > 8 || db->row_bytes < 2048 || db->n * db->row_bytes <= (96ull << 20);
 }
 
 tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d_out,
@@ -159,6 +173,16 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
   const int kernel = kernel_choice ? kernel_choice : auto_kernel(db, B);
   if (kernel_used) *kernel_used = kernel;
   cudaError_t e = cudaSuccess;
+  if (kernel == 5 && kernel_choice == 0 && db->forced_kernel == 0) {
+    // no room for the copy: the register-tiled kernel
+    e = tcopy_ensure(db, st);
+    if (e == cudaErrorMemoryAllocation)
+      return enqueue_read(db, d_req - db->req_off, B, d_out, st, d_seeds, kernel_used, 2);
+    if (e != cudaSuccess) return cuda_status(e);
+  } else if (kernel == 2 && tensor_mid(db, B)) {
+    db->mid_reads = 1;
+  }
+  if (kernel == 5 && !tensor_mid(db, B)) db->tt_wanted = true;
   if (kernel == 1 || kernel == 3) {
     const uint32_t* T = reinterpret_cast<const uint32_t*>(db->d_table);
     for (uint32_t b0 = 0; b0 < B && e == cudaSuccess; b0 += kPlainMaxB) {
@@ -325,7 +349,8 @@ tpir_status bloom_insert_core(tpir_db* db, const uint64_t* pos, uint32_t count, 
 
 // The kernel a job of a many-table launch takes: 4 Four-Russians (forced),
 // 5 tensor-core (forced, or 48 or more requests on rows of 256 bytes or
-// more), else 2 register-tiled.
+// more, or a smaller batch it is faster at on a table that has its transposed
+// copy), else 2 register-tiled.
 int multi_kernel(const tpir_read_job& q) {
   const int forced = q.db->forced_kernel;
   if (forced == 4 && q.db->Wd >= 64) return 4;
@@ -336,7 +361,9 @@ int multi_kernel(const tpir_read_job& q) {
       if (kp.kernel == 5 || (kp.kernel == 4 && q.db->Wd >= 64)) return kp.kernel;
       return 2;  // the plain kernel's jobs run in the register-tiled launch
     }
-    if (q.B >= kTensorMinB && q.db->Wd >= 64) return 5;
+    if (q.db->tt_denied) return 2;
+    if (q.B >= kTensorMinB && q.db->Wd >= kTensorMinWd) return 5;
+    if (tensor_mid(q.db, q.B) && q.db->tt_valid) return 5;
   }
   return 2;
 }
@@ -364,15 +391,14 @@ tpir_status enqueue_multi(const tpir_read_job* jobs, uint32_t njobs, cudaStream_
       (q.B > 256 ? m4w : m4).push_back(r);
     } else if (kind == 5) {
       const cudaError_t e = tcopy_ensure(q.db, st);
+      if (e == cudaErrorMemoryAllocation && q.db->forced_kernel == 0) {
+        lop3.push_back(q);  // no room for the copy
+        continue;
+      }
       if (e != cudaSuccess) return cuda_status(e);
+      if (!tensor_mid(q.db, q.B)) q.db->tt_wanted = true;
       M4Request t = r;
       t.Tt = q.db->d_tt;
-      KernelPlan kp;
-      bool exact = false;
-      if (kernel_plan_lookup(q.db->Wd, q.B, q.db->n, &kp, &exact) && kp.kernel == 5 && exact) {
-        if (kp.sched.mode == 2) t.kc_rows = kp.sched.kc_rows;
-        t.loads = kp.sched.loads;
-      }
       tc.push_back(t);
     } else {
       lop3.push_back(q);
@@ -380,7 +406,7 @@ tpir_status enqueue_multi(const tpir_read_job* jobs, uint32_t njobs, cudaStream_
   }
   tpir_status s = enqueue_multi_lop3(lop3.data(), static_cast<uint32_t>(lop3.size()), st);
   if (s == TPIR_OK && !tc.empty())
-    s = cuda_status(launch_gf2_mma_multi(tc.data(), static_cast<uint32_t>(tc.size()), st));
+    s = cuda_status(launch_gf2_tmem_multi(tc.data(), static_cast<uint32_t>(tc.size()), st));
   if (s == TPIR_OK && !m4w.empty())
     s = cuda_status(launch_m4rm_multi(m4w.data(), static_cast<uint32_t>(m4w.size()), true, st));
   if (s == TPIR_OK && !m4.empty())
@@ -859,6 +885,8 @@ tpir_status tpir_read_multi_graph_create(const tpir_read_job* jobs, uint32_t njo
     order_writes_after_reads(db, db->stream);
     cudaError_t e = cudaStreamWaitEvent(db->stream, db->last_write, 0);
     if (e == cudaSuccess) e = tcopy_ensure(db, db->stream);
+    if (e == cudaErrorMemoryAllocation && db->forced_kernel == 0) continue;  // read by another kernel
+    db->tt_wanted = true;  // replays read the copy as it then is
     if (e == cudaSuccess) e = cudaEventRecord(db->last_write, db->stream);
     if (e != cudaSuccess) {
       delete g;

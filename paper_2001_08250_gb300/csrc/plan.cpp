@@ -5,9 +5,9 @@
 // row / buckets, rows per pipeline stage) is timed on the table itself with
 // CUDA events; the fastest is cached under (row width, batch-size class) and
 // used by every later launch of that kernel.  Then the other kernels are
-// timed on the same batch -- the tensor-core kernel under each schedule
-// (spans, items of several k-chunk sizes), the Four-Russians kernel, the
-// plain kernel -- and the fastest kernel with its schedule is cached under
+// timed on the same batch -- the tensor-core kernel under each schedule (table
+// operand in tensor memory, CTA pairs, k-chunks of several sizes), the
+// Four-Russians kernel, the plain kernel -- and the fastest kernel with its schedule is cached under
 // (row width, batch-size class, table-size class): the automatic choice of
 // single-table reads, many-table launches and the serve loop follows it
 // instead of the built-in batch thresholds.  Both caches can be saved to and
@@ -183,18 +183,14 @@ tpir_status tpir_autotune(tpir_db* db, uint32_t B, uint32_t reps, tpir_tune_resu
   double best_k_us = best;
   double us_tensor = 0.0, us_m4rm = 0.0, us_plain = 0.0;
   uint32_t tensor_tried = 0;
-  if (e == cudaSuccess && db->Wd >= 64) {
+  if (e == cudaSuccess && tcopy_ensure(db, st) == cudaSuccess) {  // (no room for the copy: not tried)
     std::vector<GSched> scheds;
-    for (uint32_t loads : {0u, 1u}) {
-      if (gf2_span_ok(db->n, db->Wd, B)) scheds.push_back(GSched{1, 0, loads});
-      scheds.push_back(GSched{2, 0, loads});
-      for (uint32_t kc : {4096u, 8192u, 16384u, 32768u})
-        if (kc < (db->n + 255) / 256 * 256) scheds.push_back(GSched{2, kc, loads});
-    }
-    if (B > 128) {  // items on CTA pairs (mode 2 above) against items on single CTAs
-      scheds.push_back(GSched{3, 0, 0});
-      for (uint32_t kc : {4096u, 8192u, 16384u, 32768u})
-        if (kc < (db->n + 255) / 256 * 256) scheds.push_back(GSched{3, kc, 0});
+    // mode 1 (table operand in tensor memory) and, above 128 requests, mode 2
+    // (CTA pairs), each with planned and with given k-chunks
+    for (uint32_t mode = 1; mode <= (B > 128 ? 2u : 1u); ++mode) {
+      scheds.push_back(GSched{mode, 0, 0});
+      for (uint32_t kc : {2048u, 4096u, 8192u, 16384u, 32768u})
+        if (kc < (db->n + 255) / 256 * 256) scheds.push_back(GSched{mode, kc, 0});
     }
     for (const GSched& sc : scheds) {
       const double us = time_it([&]() {
@@ -331,7 +327,7 @@ tpir_status tpir_tune_load(const char* path) {
                     &wd, &bc, &nc, &kern, &tm, &kc, &tl) == 7) {
       // accept only choices the library can run
       if (!(kern == 1 || kern == 2 || kern == 4 || kern == 5) || tm > 3 || wd == 0 || (wd % 4) != 0 ||
-          (kern >= 4 && wd < 64) || kc > 32768 || (kc % 256) != 0 || tl > 1) {
+          (kern == 4 && wd < 64) || kc > 32768 || (kc % 256) != 0 || tl > 1) {
         rc = TPIR_EINVAL;
         continue;
       }

@@ -73,18 +73,27 @@ cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&db->d_tt), tcopy_bytes(db->n, db->row_bytes));
     if (e != cudaSuccess) {
       db->d_tt = nullptr;
+      db->tt_denied = e == cudaErrorMemoryAllocation;
+      cudaGetLastError();
       return e;
     }
   }
   TcopyBlocks all{};
-  const cudaError_t e = launch_tcopy(db, all, st);
+  cudaError_t e = launch_tcopy(db, all, st);
+  // reads on other streams come after the copy as they come after a write
+  if (e == cudaSuccess) e = cudaEventRecord(db->last_write, st);
   if (e == cudaSuccess) db->tt_valid = true;
   return e;
 }
 
 cudaError_t tcopy_after_load(tpir_db* db, cudaStream_t st) {
+  db->tt_denied = false;
   if (!db->d_tt) return cudaSuccess;  // built on first use
   db->tt_valid = false;
+  if (!db->tt_wanted) {  // only smaller batches used it: made again by the second of them
+    db->mid_reads = 0;
+    return cudaSuccess;
+  }
   return tcopy_ensure(db, st);
 }
 
@@ -97,6 +106,11 @@ cudaError_t tcopy_after_moves(tpir_db* db, const MoveOp* ops, size_t nops, cudaS
     if (ops[i].dst != kTmpSlot) kbs.push_back(ops[i].dst / db->d / 64);
   std::sort(kbs.begin(), kbs.end());
   kbs.erase(std::unique(kbs.begin(), kbs.end()), kbs.end());
+  if (!db->tt_wanted && kbs.size() > 16) {  // as after a load
+    db->tt_valid = false;
+    db->mid_reads = 0;
+    return cudaSuccess;
+  }
   if (kbs.size() > kTcopyMaxBlocks) return launch_tcopy(db, bl, st);  // rebuild it all
   bl.count = static_cast<uint32_t>(kbs.size());
   std::copy(kbs.begin(), kbs.end(), bl.kb);

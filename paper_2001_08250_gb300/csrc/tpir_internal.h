@@ -1,6 +1,7 @@
 // Internal declarations of libtalekpir (not part of the C ABI).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -83,13 +84,11 @@ static_assert(sizeof(ScanLaunch) <= 32000, "kernel parameters must stay below 32
 // Assigns the next item-counter slot (rotating).
 uint32_t next_counter_slot();
 
-// Schedule of a one-table tensor-core launch: mode 0 = planned (above 128
-// requests with TMA-staged rows: items on CTA pairs; else spans or items as
-// the cost model finds), 1 = spans (if admissible), 2 = items of kc_rows
-// buckets (0: the cost model's size; on CTA pairs above 128 requests), 3 =
-// the same items on single CTAs; loads = 1: request words loaded by the
-// expander threads instead of staged by TMA (room for a deeper ring of table
-// stages; single CTAs).
+// Schedule of a one-table tensor-core launch: mode 0 = planned (the form
+// estimated faster), 1 or 3 = table operand in tensor memory (gf2tmem.cu), 2 =
+// CTA pairs (gf2mma.cu) above 128 requests with TMA-staged rows, else as 1;
+// kc_rows = buckets per k-chunk (0: planned; cut to what the form holds);
+// loads = 1 (saved plans of request words loaded by threads): as mode 1.
 struct GSched {
   uint32_t mode = 0;
   uint32_t kc_rows = 0;
@@ -150,18 +149,24 @@ cudaError_t launch_zero_outputs(const ScanLaunch& L, cudaStream_t st);
 // them: zeros, or the masks of `seeds` (PDL-chained).
 cudaError_t launch_init_replies(uint4* out, uint32_t B, uint32_t row_u4, const uint8_t* seeds,
                                 cudaStream_t st);
-// Tensor-core batched read (gf2mma.cu): the GF(2) product as an exact integer
+// Tensor-core batched read (gf2tmem.cu; gf2mma.cu: the CTA-pair form and the
+// choice between them): the GF(2) product as an exact integer
 // product of 0/1 matrices on tcgen05 (packed e2m1 operands), reduced mod 2.
 // Tt is the table's bit-transposed copy (tcopy.cu).
 cudaError_t launch_gf2_mma(const uint64_t* Tt, uint64_t n, uint32_t Wd, const uint64_t* R,
                            uint32_t words64, uint32_t B, uint32_t* out, const uint8_t* seeds,
                            cudaStream_t st, const GSched* sched = nullptr);
-// True if span mode is admissible for this shape (at most one k-chunk of
-// stages per CTA).
-bool gf2_span_ok(uint64_t n, uint32_t Wd, uint32_t B);
+// Tensor map of a transposed table as a 2-D array of 64-bit words (row_bits
+// columns x ceil(n / 64) blocks), box `width` columns x 4 blocks.
+cudaError_t gf2_table_map(const uint64_t* Tt, uint64_t n, uint32_t Wd, uint32_t width,
+                          CUtensorMap* out);
 struct M4Request;
-// Many tables in one launch of the tensor-core kernel (up to TPIR_MAX_JOBS).
-cudaError_t launch_gf2_mma_multi(const M4Request* reqs, uint32_t count, cudaStream_t st);
+cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const uint64_t* R,
+                            uint32_t words64, uint32_t B, uint32_t* out, const uint8_t* seeds,
+                            cudaStream_t st, uint32_t kc_rows = 0);
+cudaError_t launch_gf2_tmem_multi(const M4Request* reqs, uint32_t count, cudaStream_t st);
+// Its estimated clocks on the whole device, launch included.
+double gf2_tmem_clk(uint64_t n, uint32_t Wd, uint32_t B, bool masked);
 int device_sm_count();
 int plain_ctas_per_sm();
 int batched_ctas_per_sm();
@@ -227,8 +232,6 @@ struct M4Request {
   uint32_t* out;
   const uint8_t* seeds;  // B x 32-byte mask seeds, or null
   const uint64_t* Tt = nullptr;  // tensor-core jobs: the bit-transposed table
-  uint32_t kc_rows = 0;          // tensor-core jobs: k-chunk rows (0: planned)
-  uint32_t loads = 0;            // tensor-core jobs: request words loaded by threads
 };
 cudaError_t launch_m4rm(const uint32_t* T, uint64_t n, uint32_t Wd, const uint64_t* R,
                         uint32_t words64, uint32_t B, uint32_t* out, const uint8_t* seeds,
@@ -244,7 +247,8 @@ cudaError_t launch_xor_combine(const uint4* const* srcs, uint32_t count, uint64_
 cudaError_t launch_m4rm_multi(const M4Request* reqs, uint32_t count, bool wide, cudaStream_t st);
 constexpr uint32_t kM4rmMinB = 176;  // batch from which the Four-Russians kernel beats LOP3
 constexpr uint32_t kPlainMaxB = 4;    // requests per launch of the plain kernel
-constexpr uint32_t kTensorMinB = 48;  // batch from which the tensor-core kernel beats LOP3 (measured)
+constexpr uint32_t kTensorMinWd = 64;  // row words from which it does so
+constexpr uint32_t kTensorMinB = 48;  // batch from which a read takes the tensor-core kernel at once
 cudaError_t launch_selftest_wait(uint64_t limit_ns, cudaStream_t st);
 // Rice coding of sparse bit vectors (rice.cu).
 struct RiceRequest {
@@ -374,6 +378,10 @@ struct tpir_db {
   // then kept equal to the table in stream order)
   uint64_t* d_tt = nullptr;
   bool tt_valid = false;
+  bool tt_wanted = false;  // large batches, tuned or forced reads or a captured graph use it: kept
+                           // equal to the table at every load and write
+  bool tt_denied = false;  // there was no room for it; asked for again after a load
+  uint32_t mid_reads = 0;  // 1: a batch of tensor_mid size was read without the copy
 };
 
 namespace tpir {
@@ -395,6 +403,9 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
                          int* kernel_used = nullptr, int kernel_choice = 0);
 // The kernel a read of B requests takes on db unless told otherwise.
 int auto_kernel(const tpir_db* db, uint32_t B);
+// A batch, other than the large ones on wide rows, that the tensor-core kernel
+// reads faster than the register-tiled one.
+bool tensor_mid(const tpir_db* db, uint32_t B);
 // order stream `st` after the db's last write, and record a read event
 void order_after_writes(tpir_db* db, cudaStream_t st);
 void note_read(tpir_db* db, cudaStream_t st);

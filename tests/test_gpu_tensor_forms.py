@@ -1,0 +1,85 @@
+"""GPU parity of the tensor-core read with the table operand in tensor memory:
+its block, chunk, tile and stage edges, and the batch sizes whose route
+changes once a table has its transposed copy."""
+
+import numpy as np
+import pytest
+
+import oracle
+from gpu_helpers import dev_out, require_cuda, to_dev, to_host
+from paper_2001_08250_gb300 import synth, talekpir
+
+pytestmark = pytest.mark.gpu
+
+TENSOR = 5
+
+# one column tile and several; buckets around a word (64) and a stage (256);
+# request blocks of 16 .. 128 with and without a second, third, ... block;
+# k-chunks that end within a stage; more chunks than one
+SHAPES = [
+    (1, 1, 16, 1), (64, 1, 16, 16), (65, 1, 32, 17), (255, 1, 48, 33), (257, 2, 64, 64),
+    (1000, 1, 112, 65), (2817, 1, 128, 128), (2900, 2, 64, 97), (5700, 1, 64, 113),
+    (700, 4, 256, 129), (20011, 1, 16, 70), (513, 1, 80, 300), (90001, 1, 32, 20),
+]
+
+
+@pytest.mark.parametrize("n,d,z,B", SHAPES)
+def test_tensor_memory_form_bit_exact(n, d, z, B):
+    """Plain and masked replies equal the oracle's, from request rows at an
+    8-byte offset (which only this form reads) and at a 16-byte one."""
+    require_cuda()
+    T = synth.table_bytes(n, d, z, seed=160, table=n)
+    R = synth.random_bits(B, n, seed=161, table=n)
+    S = synth.mask_seeds(B, seed=162, table=n)
+    exp = oracle.read_batch(T, n, d, z, R)
+    with talekpir.DB(n, d, z) as db:
+        db.load(T)
+        db.set_kernel(TENSOR)
+        for offset in (0, 1):
+            flat = to_dev(np.concatenate([np.zeros(offset, np.uint64), R.reshape(-1)]))
+            out = dev_out(B, d * z)
+            db.read_batch_async(flat[offset:], B, out)
+            assert np.array_equal(to_host(out), exp), offset
+        assert np.array_equal(db.read_batch_masked(R, S), oracle.read_batch_masked(T, n, d, z, R, S))
+    assert talekpir.device_status() == talekpir.OK
+
+
+@pytest.mark.parametrize("n,d,z,B", [(3000, 4, 256, 5), (3000, 4, 256, 47), (5000, 1, 64, 9),
+                                     (5000, 1, 64, 130), (300, 1, 16, 47)])
+def test_smaller_batches_before_and_after_the_transposed_copy(n, d, z, B):
+    """The first batch of these sizes runs without the transposed copy, the
+    second makes it, the third uses it; all equal the oracle's, also after a
+    load and after writes, and through many-table calls and a captured graph."""
+    torch = require_cuda()
+    R = synth.random_bits(B, n, seed=171, table=n)
+    dR = to_dev(R)
+    keys = synth.write_keys(40, seed=172)
+    b1, b2 = synth.bucket_pairs(keys, n)
+    M = synth.messages(40, z, seed=172)
+    with talekpir.DB(n, d, z) as db:
+        for load in range(2):
+            T = synth.table_bytes(n, d, z, seed=173 + load, table=n)
+            db.load(T)
+            exp = oracle.read_batch(T, n, d, z, R)
+            for _ in range(3):
+                out = dev_out(B, d * z)
+                db.read_batch_async(dR, B, out)
+                assert np.array_equal(to_host(out), exp)
+        status, _ = db.write_batch(b1, b2, M)
+        assert (status == 0).all()
+        db.sync()
+        T = db.dump()
+        exp = oracle.read_batch(T.reshape(n, d * z), n, d, z, R)
+        out = dev_out(B, d * z)
+        db.read_batch_async(dR, B, out)
+        assert np.array_equal(to_host(out), exp)
+        job = (db, B, dR, dev_out(B, d * z))
+        talekpir.read_multi_async([job])
+        assert np.array_equal(to_host(job[3]), exp)
+        job[3].zero_()
+        g = talekpir.MultiGraph([job])
+        g.launch()
+        torch.cuda.synchronize()
+        assert np.array_equal(to_host(job[3]), exp)
+        g.close()
+    assert talekpir.device_status() == talekpir.OK

@@ -1056,6 +1056,33 @@ tpir_status tpir_bloom_get_compressed(tpir_db* db, uint32_t which, int32_t k, vo
   return cuda_status(e);
 }
 
+// The library's own stream-ordered pool of the current device: it keeps up to
+// 32 MiB across synchronisations (the default pool gives everything back at
+// each, and an encode that was waited for then took 170 us more); what is above
+// that goes back.  Null: not to be had, the default pool is used.
+static cudaMemPool_t scratch_pool() {
+  static std::mutex mu;
+  static cudaMemPool_t pools[64] = {nullptr};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> g(mu);
+  if (!pools[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    uint64_t keep = 32ull << 20;
+    cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    pools[dev] = p;
+  }
+  return pools[dev];
+}
+
 tpir_status tpir_rice_encode_async(const uint64_t* d_bits, uint64_t m, int32_t k, void* d_out,
                                    uint64_t cap_bytes, uint64_t* d_result, void* stream) {
   if (!d_bits || !d_out || !d_result || m == 0 || k > 63 || (cap_bytes & 3) ||
@@ -1064,9 +1091,11 @@ tpir_status tpir_rice_encode_async(const uint64_t* d_bits, uint64_t m, int32_t k
     return TPIR_EINVAL;
   const RiceRequest rq{d_bits, m, k, static_cast<uint32_t*>(d_out), cap_bytes / 4, d_result};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // scratch from the stream-ordered allocator: calls on other streams do not share it
+  // stream-ordered scratch: calls on other streams do not share it
   void* scratch = nullptr;
-  cudaError_t e = cudaMallocAsync(&scratch, rice_scratch_bytes(m), st);
+  cudaMemPool_t pool = scratch_pool();
+  cudaError_t e = pool ? cudaMallocFromPoolAsync(&scratch, rice_scratch_bytes(m), pool, st)
+                       : cudaMallocAsync(&scratch, rice_scratch_bytes(m), st);
   if (e == cudaSuccess) e = launch_rice_encode(rq, scratch, st);
   if (scratch) {
     const cudaError_t f = cudaFreeAsync(scratch, st);

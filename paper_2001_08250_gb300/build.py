@@ -37,7 +37,7 @@ def sources() -> list[str]:
 
 def _digest() -> str:
     h = hashlib.sha256()
-    files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     files.append(os.path.join(INCLUDE, "talekpir.h"))
     for f in sorted(files):
         h.update(f.encode())

@@ -667,8 +667,10 @@ tpir_status tpir_db_load_async(tpir_db* db, const void* src, size_t bytes, void*
   order_writes_after_reads(db, st);
   cudaError_t e = cudaEventRecord(db->stream_mark, db->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, db->stream_mark, 0);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(db->d_table, src, bytes, cudaMemcpyDefault, st);
-  if (e == cudaSuccess) e = tcopy_after_load(db, st);
+  if (e == cudaSuccess && !tcopy_load(db, src, st, &e)) {
+    e = cudaMemcpyAsync(db->d_table, src, bytes, cudaMemcpyDefault, st);
+    if (e == cudaSuccess) e = tcopy_after_load(db, st);
+  }
   if (e == cudaSuccess) e = cudaEventRecord(db->last_write, st);
   if (e != cudaSuccess) return cuda_status(e);
   db->meta->clear();

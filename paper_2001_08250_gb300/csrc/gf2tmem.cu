@@ -60,6 +60,7 @@
 #include <atomic>
 #include <vector>
 
+#include "bits.cuh"
 #include "chacha.cuh"
 #include "mbar.cuh"
 #include "tpir_internal.h"
@@ -262,37 +263,6 @@ __device__ __forceinline__ uint32_t t_parities(const uint32_t (&r)[32]) {
     w = __funnelshift_r(w, __float_as_uint(__uint_as_float(r[j]) + 8388608.0f), 1);
   return w;
 }
-
-// Transposes the 32 x 32 bit matrix of a warp (lane i's word = row i): lane j
-// gets bit j of every lane, lane i's at bit i.  Five exchanges of s x s blocks:
-// s = 16 and 8 by byte selection, s = 4, 2, 1 by a rotation and a mask.
-struct TTranspose {
-  uint32_t sel16, sel8, keep4, keep2, keep1, rot4, rot2, rot1;
-  // formed anew for each tile (eight registers that the counts need)
-  __device__ __forceinline__ TTranspose() {
-    uint32_t lane;
-    asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
-    sel16 = lane & 16u ? 0x3276u : 0x5410u;
-    sel8 = lane & 8u ? 0x3715u : 0x6240u;
-    keep4 = lane & 4u ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
-    keep2 = lane & 2u ? 0xCCCCCCCCu : 0x33333333u;
-    keep1 = lane & 1u ? 0xAAAAAAAAu : 0x55555555u;
-    rot4 = lane & 4u ? 28u : 4u;
-    rot2 = lane & 2u ? 30u : 2u;
-    rot1 = lane & 1u ? 31u : 1u;
-  }
-  static __device__ __forceinline__ uint32_t step(uint32_t x, uint32_t s, uint32_t keep, uint32_t rot) {
-    const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, s);
-    return (x & keep) | (__funnelshift_l(y, y, rot) & ~keep);
-  }
-  __device__ __forceinline__ uint32_t operator()(uint32_t x) const {
-    x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 16), sel16);
-    x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 8), sel8);
-    x = step(x, 4, keep4, rot4);
-    x = step(x, 2, keep2, rot2);
-    return step(x, 1, keep1, rot1);
-  }
-};
 
 // The item's requests into shared memory: rows b0 .. b0 + mb_rows - 1 (zeros
 // past the batch), words w0 .. w1 - 1, by the reply warps (this one: w).  A warp
@@ -634,7 +604,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
           __syncwarp();
           if (lane == 0) mb::arrive(&reqf);
         }
-        const TTranspose transpose;
+        const WarpTranspose transpose;  // formed anew for each tile: its registers are the counts' before
         const uint32_t ob = out0 + (te & 1u) * kTOutBytes, oq = ob + (c0 + lane) * 16u + quarter * 4u;
         if (c0 < N)
           asm volatile("st.shared.b32 [%0], %1;" ::"r"(oq), "r"(transpose(pw0)) : "memory");

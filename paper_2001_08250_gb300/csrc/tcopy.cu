@@ -17,48 +17,78 @@
 #include <algorithm>
 #include <vector>
 
+#include "bits.cuh"
 #include "tpir_internal.h"
 
 namespace tpir {
 namespace {
 
-// One work item: block kb (64 buckets) x 8 words (256 columns) of the row.
-// Warp w takes word w: lane l holds word w of buckets 64 kb + l and
-// 64 kb + 32 + l, and 32 ballots give the word's 32 columns over the 64
-// buckets; lane j keeps column 32 w + j and stores it (32 lanes x 8 bytes,
-// contiguous).
-__global__ void __launch_bounds__(256) tcopy_kernel(const uint32_t* __restrict__ T, uint64_t n,
-                                                    uint32_t Wd, uint64_t* __restrict__ Tt,
+// One work item: block kb (64 buckets) x 32 words of the row.  The 64 x 128
+// bytes come in by whole 128-byte lines, and with COPY go out to the table (a
+// bulk load from device memory: the source is read once for both); each warp
+// then takes four words: lane l holds word w of buckets 64 kb + l and 64 kb +
+// 32 + l, and two 32 x 32 transposes in registers give lane j column 32 w + j
+// over the 64 buckets (32 lanes x 8 bytes stored, contiguous).
+// Bound by HBM: a load of 32 768 x 4 KiB takes 74 us for its three passes over
+// 128 MiB (312 and a copy of 40 before it when each warp read 32 rows' words 4 KiB
+// apart and took 64 ballots a word); 256 blocks after a batch of writes 21 (126).
+template <bool COPY>
+__global__ void __launch_bounds__(256) tcopy_kernel(const uint4* __restrict__ src, uint64_t n, uint32_t Wd,
+                                                    uint4* __restrict__ table, uint64_t* __restrict__ Tt,
                                                     uint64_t nblocks, const __grid_constant__ TcopyBlocks bl) {
+  __shared__ uint32_t tile[64][33];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t chunks = (Wd + 7) / 8;
+  const uint32_t chunks = (Wd + 31) / 32, U = Wd / 4;
   const uint64_t items = (bl.count ? bl.count : nblocks) * chunks;
   const uint64_t row_bits = static_cast<uint64_t>(Wd) * 32;
+  const WarpTranspose transpose;
   for (uint64_t it = blockIdx.x; it < items; it += gridDim.x) {
     const uint64_t kb = bl.count ? bl.kb[it / chunks] : it / chunks;
-    const uint32_t w = static_cast<uint32_t>(it % chunks) * 8 + warp;
-    if (w >= Wd) continue;  // uniform over the warp
-    const uint64_t r0 = 64 * kb + lane, r1 = r0 + 32;
-    const uint32_t x0 = r0 < n ? __ldg(T + r0 * Wd + w) : 0u;
-    const uint32_t x1 = r1 < n ? __ldg(T + r1 * Wd + w) : 0u;
-    uint64_t mine = 0;
+    const uint32_t w0 = static_cast<uint32_t>(it % chunks) * 32;
+    // thread: 16 bytes of rows threadIdx / 8 and 32 + threadIdx / 8
+    const uint32_t r = threadIdx.x >> 3, u = threadIdx.x & 7u, uc = w0 / 4 + u;
+    uint4 v[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
 #pragma unroll
-    for (uint32_t j = 0; j < 32; ++j) {
-      const uint32_t lo = __ballot_sync(0xFFFFFFFFu, (x0 >> j) & 1u);
-      const uint32_t hi = __ballot_sync(0xFFFFFFFFu, (x1 >> j) & 1u);
-      if (lane == j) mine = static_cast<uint64_t>(lo) | (static_cast<uint64_t>(hi) << 32);
+    for (uint32_t h = 0; h < 2; ++h) {
+      const uint64_t row = 64 * kb + 32 * h + r;
+      if (row < n && uc < U) v[h] = src[row * U + uc];
     }
-    Tt[kb * row_bits + static_cast<uint64_t>(w) * 32 + lane] = mine;
+    __syncthreads();  // the tile's last readers are done
+#pragma unroll
+    for (uint32_t h = 0; h < 2; ++h) {
+      uint32_t* t = &tile[32 * h + r][4 * u];
+      t[0] = v[h].x;
+      t[1] = v[h].y;
+      t[2] = v[h].z;
+      t[3] = v[h].w;
+      const uint64_t row = 64 * kb + 32 * h + r;
+      if (COPY && row < n && uc < U) table[row * U + uc] = v[h];
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i) {
+      const uint32_t c = 4 * warp + i;
+      if (w0 + c >= Wd) break;  // uniform over the warp
+      const uint32_t lo = transpose(tile[lane][c]), hi = transpose(tile[32 + lane][c]);
+      Tt[kb * row_bits + static_cast<uint64_t>(w0 + c) * 32 + lane] =
+          static_cast<uint64_t>(lo) | (static_cast<uint64_t>(hi) << 32);
+    }
   }
 }
 
-cudaError_t launch_tcopy(const tpir_db* db, const TcopyBlocks& bl, cudaStream_t st) {
+// src: the table itself, or (all blocks) device memory to copy to it as well
+cudaError_t launch_tcopy(const tpir_db* db, const void* src, const TcopyBlocks& bl, cudaStream_t st) {
   const uint64_t nblocks = (db->n + 63) / 64;
-  const uint64_t items = (bl.count ? bl.count : nblocks) * ((db->Wd + 7) / 8);
+  const uint64_t items = (bl.count ? bl.count : nblocks) * ((db->Wd + 31) / 32);
   if (items == 0) return cudaSuccess;
-  const uint64_t grid = std::min<uint64_t>(items, static_cast<uint64_t>(device_sm_count()) * 8);
-  tcopy_kernel<<<static_cast<uint32_t>(grid), 256, 0, st>>>(
-      reinterpret_cast<const uint32_t*>(db->d_table), db->n, db->Wd, db->d_tt, nblocks, bl);
+  const uint32_t grid = static_cast<uint32_t>(
+      std::min<uint64_t>(items, static_cast<uint64_t>(device_sm_count()) * 8));
+  const uint4* s4 = static_cast<const uint4*>(src);
+  uint4* t4 = reinterpret_cast<uint4*>(db->d_table);
+  if (src == db->d_table)
+    tcopy_kernel<false><<<grid, 256, 0, st>>>(s4, db->n, db->Wd, t4, db->d_tt, nblocks, bl);
+  else
+    tcopy_kernel<true><<<grid, 256, 0, st>>>(s4, db->n, db->Wd, t4, db->d_tt, nblocks, bl);
   count_launches();
   return cudaGetLastError();
 }
@@ -79,11 +109,33 @@ cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
     }
   }
   TcopyBlocks all{};
-  cudaError_t e = launch_tcopy(db, all, st);
+  cudaError_t e = launch_tcopy(db, db->d_table, all, st);
   // reads on other streams come after the copy as they come after a write
   if (e == cudaSuccess) e = cudaEventRecord(db->last_write, st);
   if (e == cudaSuccess) db->tt_valid = true;
   return e;
+}
+
+bool tcopy_load(tpir_db* db, const void* src, cudaStream_t st, cudaError_t* e) {
+  // only where the copy is rebuilt anyway, from memory of this device that the
+  // kernel can read by 16 bytes
+  if (!db->d_tt || !db->tt_wanted || (reinterpret_cast<uintptr_t>(src) & 15)) return false;
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, src) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  int dev = -1;
+  if (at.type != cudaMemoryTypeDevice || cudaGetDevice(&dev) != cudaSuccess || dev != at.device) return false;
+  const uint8_t* s8 = static_cast<const uint8_t*>(src);
+  const uint64_t bytes = db->n * db->row_bytes;
+  if (s8 < db->d_table + bytes && db->d_table < s8 + bytes) return false;  // overlapping: a plain copy
+  TcopyBlocks all{};
+  db->tt_denied = false;
+  db->tt_valid = false;
+  *e = launch_tcopy(db, src, all, st);
+  if (*e == cudaSuccess) db->tt_valid = true;
+  return true;
 }
 
 cudaError_t tcopy_after_load(tpir_db* db, cudaStream_t st) {
@@ -111,10 +163,10 @@ cudaError_t tcopy_after_moves(tpir_db* db, const MoveOp* ops, size_t nops, cudaS
     db->mid_reads = 0;
     return cudaSuccess;
   }
-  if (kbs.size() > kTcopyMaxBlocks) return launch_tcopy(db, bl, st);  // rebuild it all
+  if (kbs.size() > kTcopyMaxBlocks) return launch_tcopy(db, db->d_table, bl, st);  // rebuild it all
   bl.count = static_cast<uint32_t>(kbs.size());
   std::copy(kbs.begin(), kbs.end(), bl.kb);
-  return launch_tcopy(db, bl, st);
+  return launch_tcopy(db, db->d_table, bl, st);
 }
 
 }  // namespace tpir

@@ -390,6 +390,9 @@ namespace tpir {
 // a write's moves; each enqueued on `st` after the table's own update.
 cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st);
 cudaError_t tcopy_after_load(tpir_db* db, cudaStream_t st);
+// A bulk load from device memory with the rebuild in one pass over the source;
+// false: not such a load, nothing was done.
+bool tcopy_load(tpir_db* db, const void* src, cudaStream_t st, cudaError_t* e);
 cudaError_t tcopy_after_moves(tpir_db* db, const MoveOp* ops, size_t nops, cudaStream_t st);
 tpir_status set_error(tpir_status s);
 tpir_status cuda_status(cudaError_t e);

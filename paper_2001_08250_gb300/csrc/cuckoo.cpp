@@ -222,4 +222,52 @@ void CuckooMeta::rollback(const Undo& u) {
   rng_ = u.rng;
 }
 
+std::vector<MoveOp> settle_moves(const std::vector<MoveOp>& ops, uint32_t* nsave) {
+  // what each slot holds after the moves so far, as a write of it: kind 0 with
+  // src = the slot whose original content it is, 1 a payload, 2 zeros
+  std::unordered_map<uint64_t, size_t> at;  // slot (or kTmpSlot) -> index in `fin`
+  std::vector<MoveOp> fin;
+  at.reserve(2 * ops.size());
+  fin.reserve(ops.size());
+  for (const MoveOp& op : ops) {
+    MoveOp w{op.dst, op.src, op.kind, 0u};
+    if (op.kind == 0) {
+      const auto f = at.find(op.src);
+      if (f != at.end()) {
+        w.src = fin[f->second].src;
+        w.kind = fin[f->second].kind;
+      }
+    }
+    const auto ins = at.emplace(op.dst, fin.size());
+    if (ins.second)
+      fin.push_back(w);
+    else
+      fin[ins.first->second] = w;
+  }
+  std::vector<MoveOp> out;
+  std::unordered_map<uint64_t, uint64_t> saved;  // slot -> its saved index
+  for (const MoveOp& w : fin) {
+    if (w.dst == kTmpSlot || w.kind != 0 || w.src == w.dst) continue;
+    const auto f = at.find(w.src);
+    if (f == at.end()) continue;  // nothing is written there
+    const MoveOp& o = fin[f->second];
+    if (o.kind == 0 && o.src == w.src) continue;  // it keeps its content
+    if (saved.emplace(w.src, saved.size()).second) out.push_back(MoveOp{saved.size() - 1, w.src, 4u, 0u});
+  }
+  *nsave = static_cast<uint32_t>(out.size());
+  for (const MoveOp& w : fin) {
+    if (w.dst == kTmpSlot || (w.kind == 0 && w.src == w.dst)) continue;
+    MoveOp o = w;
+    if (w.kind == 0) {
+      const auto f = saved.find(w.src);
+      if (f != saved.end()) {
+        o.kind = 3;
+        o.src = f->second;
+      }
+    }
+    out.push_back(o);
+  }
+  return out;
+}
+
 }  // namespace tpir

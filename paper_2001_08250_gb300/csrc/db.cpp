@@ -279,22 +279,25 @@ tpir_status apply_writes_core(tpir_db* db, uint32_t count, const uint64_t* b1, c
       e = launch_apply_moves_param(db->d_table, db->z, m, db->d_tmp, st);
       if (e == cudaSuccess) e = tcopy_after_moves(db, ops.data(), ops.size(), st);
     } else {
-      const uint64_t ops_bytes = ops.size() * sizeof(MoveOp);
+      uint32_t nsave = 0;
+      const std::vector<MoveOp> settled = settle_moves(ops, &nsave);
+      const uint64_t ops_bytes = settled.size() * sizeof(MoveOp), save_bytes = nsave * z;
       if (!grow_pinned(reinterpret_cast<void**>(&stg.h), &stg.h_cap, pay_bytes + ops_bytes) ||
           !grow_dev(reinterpret_cast<void**>(&stg.d_payload), &stg.pay_cap, pay_bytes) ||
           !grow_dev(reinterpret_cast<void**>(&stg.d_ops), &stg.ops_cap, ops_bytes) ||
+          !grow_dev(reinterpret_cast<void**>(&stg.d_saved), &stg.saved_cap, save_bytes) ||
           (!stg.done && cudaEventCreateWithFlags(&stg.done, cudaEventDisableTiming) != cudaSuccess)) {
         take_back();
         return TPIR_ENOMEM;
       }
       std::memcpy(stg.h, msgs, pay_bytes);
-      std::memcpy(stg.h + pay_bytes, ops.data(), ops_bytes);
+      std::memcpy(stg.h + pay_bytes, settled.data(), ops_bytes);
       e = cudaMemcpyAsync(stg.d_payload, stg.h, pay_bytes, cudaMemcpyHostToDevice, st);
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(stg.d_ops, stg.h + pay_bytes, ops_bytes, cudaMemcpyHostToDevice, st);
       if (e == cudaSuccess)
-        e = launch_apply_moves(db->d_table, db->z, stg.d_ops, static_cast<uint32_t>(ops.size()),
-                               stg.d_payload, db->d_tmp, st);
+        e = launch_settled_moves(db->d_table, db->z, stg.d_ops, nsave,
+                                 static_cast<uint32_t>(settled.size()), stg.d_payload, stg.d_saved, st);
       if (e == cudaSuccess) e = cudaEventRecord(stg.done, st);
       if (e == cudaSuccess) e = tcopy_after_moves(db, ops.data(), ops.size(), st);
     }
@@ -475,6 +478,7 @@ void tpir_write_staging_release(tpir_write_staging& s) {
   if (s.h) cudaFreeHost(s.h);
   cudaFree(s.d_payload);
   cudaFree(s.d_ops);
+  cudaFree(s.d_saved);
   cudaFree(s.d_pos);
   if (s.done) cudaEventDestroy(s.done);
   s = tpir_write_staging();

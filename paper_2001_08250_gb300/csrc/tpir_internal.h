@@ -175,12 +175,19 @@ int batched_ctas_per_sm();
 struct MoveOp {   // one step of a write's slot moves, executed in order
   uint64_t dst;   // slot index (bucket*d + j), or kTmpSlot
   uint64_t src;   // slot index, kTmpSlot, or payload index (kind 1)
-  uint32_t kind;  // 0 copy slot->slot, 1 payload->slot, 2 zero slot
+  uint32_t kind;  // 0 copy slot->slot, 1 payload->slot, 2 zero slot; settled lists
+                  // also 3 saved slot->slot, 4 slot->saved slot
   uint32_t pad;
 };
 constexpr uint64_t kTmpSlot = ~0ull;
-cudaError_t launch_apply_moves(uint8_t* table, uint32_t z, const MoveOp* ops, uint32_t nops,
-                               const uint8_t* payloads, uint8_t* tmp, cudaStream_t st);
+// An ordered move list as independent ones: first the slots to save (kind 4,
+// *nsave of them: original contents that another slot takes and that are
+// overwritten), then one write for each slot whose content changes.
+std::vector<MoveOp> settle_moves(const std::vector<MoveOp>& ops, uint32_t* nsave);
+// Settled moves (ops: device list, the nsave saving ones first).
+cudaError_t launch_settled_moves(uint8_t* table, uint32_t z, const MoveOp* ops, uint32_t nsave,
+                                 uint32_t nops, const uint8_t* payloads, uint8_t* saved,
+                                 cudaStream_t st);
 // A small batch of writes with its moves and new messages in the kernel
 // parameters (no staging): at most OPS moves and BYTES of messages (payload
 // index i = bytes i*z .. of `payload`).  Two sizes: the launch copies the whole
@@ -322,6 +329,8 @@ struct tpir_write_staging {
   uint64_t pay_cap = 0;
   tpir::MoveOp* d_ops = nullptr;
   uint64_t ops_cap = 0;
+  uint8_t* d_saved = nullptr;  // slots saved by settled moves
+  uint64_t saved_cap = 0;
   uint64_t* d_pos = nullptr;
   uint64_t pos_cap = 0;
   cudaEvent_t done = nullptr;  // recorded after the last work that read the staging

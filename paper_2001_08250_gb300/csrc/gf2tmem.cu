@@ -36,23 +36,25 @@
 //   warps 0, 1    stream the raw stages: 4 words (256 buckets) of a tile's 128
 //                 columns by 2-D TMA;
 //   warps 2, 3    issue the MMAs;
-//   8 warps       table expanders, four per stream (lane quarter = warp % 4);
+//   8 or 16 warps table expanders, one or two groups of four per stream (lane
+//                 quarter = warp % 4; TLayout);
 //   8 warps       expand the item's requests, then take the tiles in order:
 //                 read the counts (tcgen05.ld), keep their parities, transpose
 //                 them into reply words, and store or XOR-reduce those.
-// Tensor memory: per stream one accumulator of 128 columns (two of 64 where no
-// block holds more than 64 requests) and three table stages of 32 columns; the
-// scale factors in the last 32.  Every wait is bounded; a wait that gives up
-// sets the status word, and the CTA drains its MMAs and TMA loads and frees its
-// tensor memory before it returns.
+// Tensor memory: per stream one accumulator of 128 (or 112) columns (used as
+// two where no block holds more than 64 (or 48) requests) and three (or four)
+// table stages of 32 columns; the scale factors in the last 32.  Every wait is
+// bounded; a wait that gives up sets the status word, and the CTA drains its MMAs
+// and TMA loads and frees its tensor memory before it returns.
 //
 // Measured (us a launch; before: both operands in shared memory, one CTA an
-// SM): 32 768 x 4 KiB: 39 at 32 requests (68 on the register-tiled kernel),
-// 40 at 64 (77), 46 at 128 (77); 50 021 x 4 160 bytes masked: 80 at 100
-// requests (135); 200 003 x 128 bytes: 13 at 64 (93 on the register-tiled
-// kernel).  What bounds it: the two issuers' and the expanders' instruction
-// latency (issue slots 55 % used, ALU pipe 53 %, tensor pipe 53 % at 128
-// requests, HBM 40 % at 16).
+// SM): 32 768 x 4 KiB: 33 at 32 requests (68 on the register-tiled kernel), 36
+// at 64 (77), 42 at 112, 45 at 128 (77); 50 021 x 4 160 bytes masked: 66 at 100
+// requests (134); 200 003 x 128 bytes: 12 at 64 (93 on the register-tiled
+// kernel).  Blocks of up to 112 requests with one expander group: 39, 40, 44 and
+// 80, 12.4.  What bounds it: instruction latency and the ALU pipe in the
+// expanders and the issuers (issue slots 55 % used, ALU pipe 53 %, tensor pipe 53 %
+// at 128 requests; HBM 60 % at 32).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -72,25 +74,38 @@ constexpr uint32_t kTCols = 128;               // table columns per tile (MMA M)
 constexpr uint32_t kTStageWords = 4;           // 64-bucket words per stage
 constexpr uint32_t kTRawBytes = kTCols * kTStageWords * 8;  // 4 KiB
 constexpr uint32_t kTStreams = 2;              // independent tile pipelines of a CTA
-constexpr uint32_t kTRaw = 5;                  // raw stages in flight per stream
-constexpr uint32_t kTResBytes = 176 * 1024;    // expanded requests of an item
-constexpr uint32_t kTOutBytes = 128 * 16;      // a tile's reply words: 16 bytes per request
-constexpr uint32_t kTOut0 = kTResBytes + kTStreams * kTRaw * kTRawBytes;
-constexpr uint32_t kTSmem = 1024 + kTOut0 + 2 * kTOutBytes;
-static_assert(kTSmem <= 231424, "dynamic shared memory above 227 KiB less the static part");
 constexpr uint32_t kTMaxN = 128;               // requests per block
-constexpr uint32_t kTSlots = 3;                // table stages in tensor memory, per stream
+constexpr uint32_t kTAccHalf = 64;             // columns to a stream's second accumulator
 constexpr uint32_t kTSlotCols = 8 * kTStageWords;
-constexpr uint32_t kTACol = kTStreams * kTMaxN;  // first column of the table rings
+constexpr uint32_t kTOutBytes = 128 * 16;      // a tile's reply words: 16 bytes per request
 constexpr uint32_t kTSfa = 480, kTSfb = 496;   // scale factors
-static_assert(kTACol + kTStreams * kTSlots * kTSlotCols <= kTSfa, "tensor memory columns overlap");
 constexpr uint32_t kTTmemCols = 512;
-constexpr uint32_t kTGroups = 1;               // expander groups of four warps, per stream
 constexpr uint32_t kTIssueWarp0 = kTStreams;   // after one TMA warp per stream
 constexpr uint32_t kTExpWarp0 = 2 * kTStreams;
-constexpr uint32_t kTEpiWarp0 = kTExpWarp0 + 4 * kTGroups * kTStreams, kTEpiWarps = 8;
+constexpr uint32_t kTEpiWarps = 8;
 static_assert(kTExpWarp0 % 4 == 0, "a warp reads the tensor-memory lanes of its quarter");
-constexpr int kTThreads = 32 * (kTEpiWarp0 + kTEpiWarps);
+
+// The two layouts of a CTA (with one group a stage's expansion, some 600 clocks
+// of dependent instructions, bounded the blocks that the MMAs do not).  G = 1: blocks of up to 128 requests, one group of
+// four expander warps per stream.  G = 2: blocks of up to 112 requests, whose
+// accumulators leave room for a fourth table stage per stream, and two groups
+// that take alternate stages; the rings are of even length, so that a slot
+// always belongs to the same group.
+template <int G>
+struct TLayout {
+  static constexpr uint32_t kRaw = G == 1 ? 5 : 6;           // raw stages in flight, per stream
+  static constexpr uint32_t kSlots = G == 1 ? 3 : 4;         // table stages in tensor memory, per stream
+  static constexpr uint32_t kAcc = G == 1 ? 128 : 112;       // accumulator columns per stream
+  static constexpr uint32_t kRes = (G == 1 ? 176 : 168) * 1024;  // expanded requests of an item
+  static constexpr uint32_t kACol = kTStreams * kAcc;        // first column of the table rings
+  static constexpr uint32_t kEpiWarp0 = kTExpWarp0 + 4 * G * kTStreams;
+  static constexpr int kThreads = 32 * (kEpiWarp0 + kTEpiWarps);
+  static constexpr uint32_t kOut0 = kRes + kTStreams * kRaw * kTRawBytes;
+  static constexpr uint32_t kSmem = 1024 + kOut0 + 2 * kTOutBytes;
+  static_assert(kSmem <= 231424, "dynamic shared memory above 227 KiB less the static part");
+  static_assert(kACol + kTStreams * kSlots * kTSlotCols <= kTSfa, "tensor memory columns overlap");
+  static_assert(kRaw % G == 0 && kSlots % G == 0, "a ring slot belongs to one group");
+};
 constexpr uint64_t kTWaitNs = 4000000000ull;
 
 struct TJob {
@@ -113,7 +128,7 @@ struct TLaunch {
   CUtensorMap maps[NJ];
   TJob jobs[NJ];
   uint32_t njobs, total_items;
-  uint32_t nbuf;  // accumulators per stream: 2 when every job's blocks hold at most 64 requests
+  uint32_t nbuf;  // accumulators per stream: 2 when every job's blocks fit half of one
 };
 constexpr int kTMultiJobs = 64;  // jobs per many-table launch (kernel parameter space)
 static_assert(sizeof(TLaunch<kTMultiJobs>) <= 32000, "kernel parameters must stay below 32 KB");
@@ -157,22 +172,23 @@ __device__ __forceinline__ bool t_item(const TLaunch<NJ>& L, uint32_t r, TItem& 
 // Shared-memory matrix descriptor of one K = 64 step of the N operand: K-major
 // without swizzle, 8-row x 16-byte core matrices, 128 bytes apart along K, 256
 // along N; the steps of a chunk are 32 N bytes apart.
-__device__ __forceinline__ uint64_t t_desc(uint32_t addr) {
-  return static_cast<uint64_t>((addr >> 4) & 0x3FFFu) | (static_cast<uint64_t>(128 >> 4) << 16) |
-         (static_cast<uint64_t>(256 >> 4) << 32) | (1ull << 46);
+// (The lower half holds the address and the distance along K.)
+constexpr uint32_t kTDescHi = (256u >> 4) | (1u << 14);
+__device__ __forceinline__ uint32_t t_desc(uint32_t addr) {
+  return ((addr >> 4) & 0x3FFFu) | (static_cast<uint32_t>(128 >> 4) << 16);
 }
 
 // D (+)= A x B.  Whether D is accumulated is a compile-time constant: back to
 // back and with fixed operands an MMA then takes its thread 12 clocks to issue,
 // 51 with the predicate formed at run time.
 template <bool ACC>
-__device__ __forceinline__ void t_mma(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void t_mma(uint32_t d, uint32_t a, uint32_t bdesc, uint32_t idesc,
                                       uint32_t sfa, uint32_t sfb) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %6, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], [%1], %2, %3, [%4], [%5], "
+      "{\n\t.reg .pred p;\n\t.reg .b64 q;\n\tsetp.ne.b32 p, %7, 0;\n\tmov.b64 q, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], [%1], q, %4, [%5], [%6], "
       "p;\n\t}" ::"r"(d),
-      "r"(a), "l"(bdesc), "r"(idesc), "r"(sfa), "r"(sfb), "n"(ACC ? 1 : 0)
+      "r"(a), "r"(bdesc), "r"(kTDescHi), "r"(idesc), "r"(sfa), "r"(sfb), "n"(ACC ? 1 : 0)
       : "memory");
 }
 
@@ -239,6 +255,13 @@ __device__ __forceinline__ void t_store_stage(uint32_t taddr, const uint64_t (&x
       : "memory");
 }
 
+// The four words of this thread's column in a raw stage.
+__device__ __forceinline__ void t_read_raw(uint32_t addr, uint64_t (&x)[4]) {
+#pragma unroll
+  for (uint32_t i = 0; i < 4; ++i)
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(x[i]) : "r"(addr + i * (kTCols * 8)) : "memory");
+}
+
 // 32 accumulator columns of this thread's lane (in registers after t_wait_ld).
 __device__ __forceinline__ void t_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -303,9 +326,12 @@ __device__ __forceinline__ void t_load_requests(const TJob& J, const TItem& it, 
   }
 }
 
-template <int NJ>
-__global__ void __launch_bounds__(kTThreads, 1)
+template <int NJ, int G>
+__global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
     gf2_tmem_kernel(const __grid_constant__ TLaunch<NJ> L, int* status) {
+  using Y = TLayout<G>;
+  constexpr uint32_t kTRaw = Y::kRaw, kTSlots = Y::kSlots, kTACol = Y::kACol, kTEpiWarp0 = Y::kEpiWarp0;
+  constexpr uint32_t kTResBytes = Y::kRes, kTOut0 = Y::kOut0, kTAcc = Y::kAcc;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[kTStreams][kTSlots], empty[kTStreams][kTSlots];
   __shared__ __align__(8) uint64_t raw_full[kTStreams][kTRaw], raw_empty[kTStreams][kTRaw];
@@ -323,7 +349,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   if (threadIdx.x == 0) {
     for (uint32_t g = 0; g < kTStreams; ++g) {
       for (uint32_t s = 0; s < kTSlots; ++s) {
-        mb::init(&full[g][s], 4);  // the four warps of one expander group
+        mb::init(&full[g][s], 4);  // the stream's four expander warps
         mb::init(&empty[g][s], 1);
       }
       for (int b = 0; b < 2; ++b) {
@@ -422,7 +448,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
     const uint32_t utmem = __shfl_sync(0xFFFFFFFFu, tmem, 0);
     const uint32_t sfa = utmem + kTSfa, sfb = utmem + kTSfb;
     const uint32_t a0 = utmem + kTACol + g * (kTSlots * kTSlotCols);
-    const uint64_t bd0 = t_desc(__shfl_sync(0xFFFFFFFFu, res0, 0));
+    const uint32_t bd0 = t_desc(__shfl_sync(0xFFFFFFFFu, res0, 0));
     const uint32_t nb2 = L.nbuf == 2 ? 1u : 0u;
     uint32_t is = 0, iph = 0;  // ring slot and its phase
     uint32_t tc = 0;           // this stream's tiles so far
@@ -432,17 +458,17 @@ __global__ void __launch_bounds__(kTThreads, 1)
       const uint32_t N = L.jobs[it.job].mb_rows;
       // A and B e2m1 (1), both K-major, UE8M0 scales (bit 23), M = 128
       const uint32_t idesc = (1u << 7) | (1u << 10) | ((N >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24);
-      const uint64_t dstep = (32u * N) >> 4;
+      const uint32_t dstep = (32u * N) >> 4;
       if (!t_wait_warp(&reqf, r & 1u, abort_flag, status)) break;
       const uint32_t W = it.w1 - it.w0;
       for (uint32_t i = g; ok && i < it.nt; i += kTStreams, ++tc) {
-        const uint32_t buf = nb2 & tc, acc = utmem + g * kTMaxN + buf * (kTMaxN / 2);
+        const uint32_t buf = nb2 & tc, acc = utmem + g * kTAcc + buf * kTAccHalf;
         const uint32_t use = tc >> nb2;  // times this accumulator was used before
         if (use && !t_wait_warp(&acce[g][buf], (use - 1u) & 1u, abort_flag, status)) {
           ok = false;
           break;
         }
-        uint64_t bd = bd0;
+        uint32_t bd = bd0;
         for (uint32_t w = 0; w < W; w += kTStageWords) {
           if (!t_wait_warp(&full[g][is], iph, abort_flag, status)) {
             ok = false;
@@ -487,65 +513,56 @@ __global__ void __launch_bounds__(kTThreads, 1)
     // ------------------------ table expanders ------------------------
     // lane = column 32 quarter + lane of the tile; every stage is expanded in
     // full (words past the chunk are not multiplied)
-    const uint32_t e = (warp - kTExpWarp0) >> 2, g = e % kTStreams, group = e / kTStreams;
-    const uint32_t quarter = warp & 3u;
+    const uint32_t e = (warp - kTExpWarp0) >> 2, g = e % kTStreams, group = e / kTStreams, quarter = warp & 3u;
     const uint32_t raw0 = res0 + kTResBytes + g * (kTRaw * kTRawBytes) + (32u * quarter + lane) * 8u;
     const uint32_t tlane = tmem + ((32u * quarter) << 16) + kTACol + g * (kTSlots * kTSlotCols);
-    uint32_t seq = 0, mine = group;  // the stream's stages through this item; this group's next
-    uint32_t rs = group, rph = 0, sl = group, ph = 0;  // its ring slots and their phases
-    // The barriers of the next stage are asked while this one is expanded and
-    // the answers used after it: asking takes about 90 clocks, and asked in turn
-    // the two bounded the pipeline.
-    bool raw_ready = false, slot_ready = false;
+    uint32_t total = 0;  // the stream's stages
     TItem it;
-    bool ok = true;
-    for (uint32_t r = 0; ok && t_item(L, r, it); ++r) {
-      seq += ((it.nt + kTStreams - 1 - g) / kTStreams) *
-             ((it.w1 - it.w0 + kTStageWords - 1) / kTStageWords);
-      for (; mine < seq; mine += kTGroups) {
-        if (!raw_ready && !mb::wait(&raw_full[g][rs], rph, abort_flag, status, kTWaitNs)) {
-          ok = false;
-          break;
-        }
-        __syncwarp();
-        uint64_t x[4];
-#pragma unroll
-        for (uint32_t i = 0; i < 4; ++i)
-          asm volatile("ld.shared.b64 %0, [%1];"
-                       : "=l"(x[i])
-                       : "r"(raw0 + rs * kTRawBytes + i * (kTCols * 8))
-                       : "memory");
-        const uint32_t rs0 = rs, s0 = sl;
-        rs += kTGroups;
-        if (rs >= kTRaw) {
-          rs -= kTRaw;
-          rph ^= 1u;
-        }
-        raw_ready = mb::test(&raw_full[g][rs], rph);
-        {
-          // the raw slot goes back once the words are in registers and ordered
-          // before the async proxy's next write to it
-          asm volatile("fence.proxy.async.shared::cta;" ::"l"(x[0]), "l"(x[1]), "l"(x[2]), "l"(x[3]) : "memory");
-          __syncwarp();
-          if (lane == 0) mb::arrive(&raw_empty[g][rs0]);
-        }
-        if (!slot_ready && !mb::wait(&empty[g][sl], ph ^ 1u, abort_flag, status, kTWaitNs)) {
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        __syncwarp();
-        t_store_stage(tlane + s0 * kTSlotCols, x);
-        sl += kTGroups;
-        if (sl >= kTSlots) {
-          sl -= kTSlots;
-          ph ^= 1u;
-        }
-        slot_ready = mb::test(&empty[g][sl], ph ^ 1u);
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mb::arrive(&full[g][s0]);
+    for (uint32_t r = 0; t_item(L, r, it); ++r)
+      total += ((it.nt + kTStreams - 1 - g) / kTStreams) *
+               ((it.w1 - it.w0 + kTStageWords - 1) / kTStageWords);
+    // One set of warps waits for every phase of a ring slot in order (a phase's
+    // parity says nothing while the phase before it is still open).  The next
+    // stage's barriers are asked and its words read while this one is stored:
+    // asking takes about 90 clocks, and in turn they bounded the pipeline.
+    uint32_t rs = group, rph = 0, sl = group, ph = 0;  // ring slots and their phases
+    bool slot_ready = false, ok = true;
+    uint64_t x[4];
+    if (group < total) {
+      ok = mb::wait(&raw_full[g][rs], 0, abort_flag, status, kTWaitNs);
+      t_read_raw(raw0 + rs * kTRawBytes, x);
+    }
+    for (uint32_t m = group; ok && m < total; m += G) {
+      __syncwarp();
+      // the raw slot goes back once the words are in registers and ordered
+      // before the async proxy's next write to it
+      asm volatile("fence.proxy.async.shared::cta;" ::"l"(x[0]), "l"(x[1]), "l"(x[2]), "l"(x[3]) : "memory");
+      __syncwarp();
+      if (lane == 0) mb::arrive(&raw_empty[g][rs]);
+      if ((rs += G) >= kTRaw) {
+        rs -= kTRaw;
+        rph ^= 1u;
+      }
+      const bool more = m + G < total;
+      const bool next = more && mb::test(&raw_full[g][rs], rph);
+      if (!slot_ready && !mb::wait(&empty[g][sl], ph ^ 1u, abort_flag, status, kTWaitNs)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      __syncwarp();
+      t_store_stage(tlane + sl * kTSlotCols, x);
+      if (next) t_read_raw(raw0 + rs * kTRawBytes, x);
+      const uint32_t s0 = sl;
+      if ((sl += G) >= kTSlots) {
+        sl -= kTSlots;
+        ph ^= 1u;
+      }
+      slot_ready = mb::test(&empty[g][sl], ph ^ 1u);
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mb::arrive(&full[g][s0]);
+      if (more && !next) {
+        if (!mb::wait(&raw_full[g][rs], rph, abort_flag, status, kTWaitNs)) break;
+        t_read_raw(raw0 + rs * kTRawBytes, x);
       }
     }
   } else {
@@ -584,8 +601,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         __syncwarp();
         uint32_t pw0, pw1 = 0;  // parities of this column, 32 requests a word
-        const uint32_t acc = tmem + ((32u * quarter) << 16) + g * kTMaxN + buf * (kTMaxN / 2) + c0;
-        {
+        const uint32_t acc = tmem + ((32u * quarter) << 16) + g * kTAcc + buf * kTAccHalf + c0;
+        if constexpr (G == 1) {
           uint32_t r0[32], r1[32];
           t_ld32(acc, r0);  // (columns past N: not used)
           if (two) t_ld32(acc + 32, r1);
@@ -595,6 +612,22 @@ __global__ void __launch_bounds__(kTThreads, 1)
           if (lane == 0) mb::arrive(&acce[g][buf]);
           pw0 = t_parities(r0);
           if (two) pw1 = t_parities(r1);
+        } else {  // (fewer registers a thread)
+          uint32_t r0[32];
+          t_ld32(acc, r0);
+          t_wait_ld();
+          if (two) {
+            pw0 = t_parities(r0);
+            t_ld32(acc + 32, r0);
+            t_wait_ld();
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mb::arrive(&acce[g][buf]);
+          if (two)
+            pw1 = t_parities(r0);
+          else
+            pw0 = t_parities(r0);
         }
         if (more && i + 1 == it.nt) {
           // every tile's MMAs have read the item's requests: the next item's
@@ -661,15 +694,18 @@ __global__ void gf2_tmem_init_kernel(const __grid_constant__ TLaunch<NJ> L) {
                blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x);
 }
 
-// Clocks of an item: W words (K = 64 steps) of nt tiles at N requests.  The two
-// streams together run a step in 0.54 N clocks (the MMA) or 52 (two issuing
-// threads, or the table words from HBM); one alone in 105, and it stands
-// still while a tile's counts are read.
+// Blocks of up to 112 requests take the layout with two expander groups.
+int t_groups(uint32_t N) { return N <= TLayout<2>::kAcc ? 2 : 1; }
+// Clocks of an item: W words (K = 64 steps, whole stages of four) of nt tiles at
+// N requests, as measured.  The two streams together run a step in 0.54 N
+// clocks (the MMA) or 45 to 52 (instruction latency); one alone in about 100,
+// and it stands still while a tile's counts are read.
 double t_item_clk(uint32_t N, uint32_t W, uint32_t nt) {
-  const double step = std::max(0.54 * N, 52.0);
-  const double both = nt * (W * step + 40.0);
-  const double one = ((nt + 1) / 2) * (W * 105.0 + (N <= kTMaxN / 2 ? 400.0 : 400.0 + 10.0 * N));
-  return 3000.0 + 0.3 * N * W + std::max(both, one);
+  const bool two = t_groups(N) == 2;
+  const double steps = (W + 3) / 4 * 4;
+  const double both = nt * (steps * std::max(0.54 * N, two ? 45.0 : 52.0) + 40.0);
+  const double one = ((nt + 1) / 2) * (steps * (two ? 95.0 : 115.0) + (N <= kTAccHalf ? 400.0 : 400.0 + 10.0 * N));
+  return 4000.0 + 0.3 * N * W + std::max(both, one);
 }
 
 TJob t_job(const uint64_t* R, uint32_t words64, uint32_t B, uint32_t* out, const uint8_t* seeds,
@@ -689,7 +725,7 @@ TJob t_job(const uint64_t* R, uint32_t words64, uint32_t B, uint32_t* out, const
   return j;
 }
 
-uint32_t t_max_words(uint32_t N) { return kTResBytes / (32 * N); }
+uint32_t t_max_words(uint32_t N) { return (t_groups(N) == 2 ? TLayout<2>::kRes : TLayout<1>::kRes) / (32 * N); }
 
 void t_set_chunks(TJob& j, uint32_t kc_words, uint32_t splits) {
   j.kc_words = kc_words;
@@ -730,34 +766,39 @@ double t_plan(TJob& j, uint32_t grid) {
   return best;
 }
 
-template <int NJ>
+template <int NJ, int G>
 cudaError_t t_launch(TLaunch<NJ>& L, cudaStream_t st) {
-  static std::atomic<bool> ready{false};
+  using Y = TLayout<G>;
+  static std::atomic<bool> ready{false};  // idempotent set-up: a race only repeats it
   if (!ready.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gf2_tmem_kernel<NJ>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kTSmem);
+    cudaError_t e = cudaFuncSetAttribute(gf2_tmem_kernel<NJ, G>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Y::kSmem);
     if (e != cudaSuccess) return e;
     ready.store(true, std::memory_order_release);
   }
   int* status = device_status_word();
   if (!status) return cudaErrorInvalidSymbol;
+  // two accumulators per stream where every block's requests fit beside others
   bool any = false;
-  for (uint32_t i = 0; i < L.njobs; ++i) any |= L.jobs[i].split == 1;
+  L.nbuf = 2u;
+  for (uint32_t i = 0; i < L.njobs; ++i) {
+    any |= L.jobs[i].split == 1;
+    if (L.jobs[i].mb_rows > Y::kAcc - kTAccHalf) L.nbuf = 1u;
+  }
   cudaError_t e = cudaSuccess;
   if (any) e = launch_pdl(gf2_tmem_init_kernel<NJ>, dim3(64, L.njobs), dim3(256), 0, st, L);
   if (e != cudaSuccess) return e;
   const uint32_t grid = std::min<uint32_t>(L.total_items, device_sm_count());
-  return launch_pdl(gf2_tmem_kernel<NJ>, dim3(grid), dim3(kTThreads), kTSmem, st, L, status);
+  return launch_pdl(gf2_tmem_kernel<NJ, G>, dim3(grid), dim3(Y::kThreads), Y::kSmem, st, L, status);
 }
 
 }  // namespace
 
-// (measured launches: 1.1 to 1.2 times the planned clocks, and 1 us, 4 with the
-// replies' initialisation before them)
+// (with a launch, and the replies' initialisation where there is one)
 double gf2_tmem_clk(uint64_t n, uint32_t Wd, uint32_t B, bool masked) {
   TJob j = t_job(nullptr, 0, B, nullptr, nullptr, n, Wd);
   const double clk = t_plan(j, static_cast<uint32_t>(device_sm_count()));
-  return 1.17 * clk + (j.split || masked ? 8000.0 : 2000.0);
+  return clk + (j.split || masked ? 8500.0 : 3000.0);
 }
 
 cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const uint64_t* R,
@@ -773,11 +814,10 @@ cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const u
   const uint64_t items = static_cast<uint64_t>(J.mbs) * J.kcs * J.splits;
   if (items > 0xFFFFFFFFull) return cudaErrorInvalidValue;
   L.total_items = static_cast<uint32_t>(items);
-  L.nbuf = J.mb_rows <= kTMaxN / 2 ? 2u : 1u;
   L.jobs[0] = J;
   const cudaError_t e = gf2_table_map(Tt, n, Wd, kTCols, &L.maps[0]);
   if (e != cudaSuccess) return e;
-  return t_launch<1>(L, st);
+  return t_groups(J.mb_rows) == 2 ? t_launch<1, 2>(L, st) : t_launch<1, 1>(L, st);
 }
 
 // Up to kTMultiJobs jobs in one persistent launch: k-chunks as long as they
@@ -788,7 +828,7 @@ static cudaError_t t_launch_multi(const M4Request* reqs, uint32_t count, cudaStr
   std::vector<TJob> js;
   std::vector<const M4Request*> src;
   double total = 0.0;
-  bool all_small = true;
+  int groups = 2;  // one layout for all jobs
   for (uint32_t i = 0; i < count; ++i) {
     const M4Request& q = reqs[i];
     if (q.B == 0) continue;
@@ -797,7 +837,7 @@ static cudaError_t t_launch_multi(const M4Request* reqs, uint32_t count, cudaStr
     const uint32_t c = t_min_chunks(j);
     t_set_chunks(j, (j.nw + c - 1) / c, 1);
     total += static_cast<double>(j.mbs) * j.kcs * t_item_clk(j.mb_rows, j.kc_words, j.tiles);
-    all_small &= j.mb_rows <= kTMaxN / 2;
+    groups = std::min(groups, t_groups(j.mb_rows));
     js.push_back(j);
     src.push_back(&q);
   }
@@ -816,7 +856,6 @@ static cudaError_t t_launch_multi(const M4Request* reqs, uint32_t count, cudaStr
   std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return cost[a] > cost[b]; });
   TLaunch<kTMultiJobs> L{};
   L.njobs = 0;
-  L.nbuf = all_small ? 2u : 1u;
   uint64_t items = 0;
   for (size_t oi : order) {
     TJob j = js[oi];
@@ -828,7 +867,7 @@ static cudaError_t t_launch_multi(const M4Request* reqs, uint32_t count, cudaStr
     L.jobs[L.njobs++] = j;
   }
   L.total_items = static_cast<uint32_t>(items);
-  return t_launch<kTMultiJobs>(L, st);
+  return groups == 2 ? t_launch<kTMultiJobs, 2>(L, st) : t_launch<kTMultiJobs, 1>(L, st);
 }
 
 cudaError_t launch_gf2_tmem_multi(const M4Request* reqs, uint32_t count, cudaStream_t st) {

@@ -173,6 +173,7 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
   const int kernel = kernel_choice ? kernel_choice : auto_kernel(db, B);
   if (kernel_used) *kernel_used = kernel;
   cudaError_t e = cudaSuccess;
+  if (kernel == 5 && (!tensor_mid(db, B) || db->forced_kernel)) db->tt_wanted = true;
   if (kernel == 5 && kernel_choice == 0 && db->forced_kernel == 0) {
     // no room for the copy: the register-tiled kernel
     e = tcopy_ensure(db, st);
@@ -182,7 +183,6 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
   } else if (kernel == 2 && tensor_mid(db, B)) {
     db->mid_reads = 1;
   }
-  if (kernel == 5 && !tensor_mid(db, B)) db->tt_wanted = true;
   if (kernel == 1 || kernel == 3) {
     const uint32_t* T = reinterpret_cast<const uint32_t*>(db->d_table);
     for (uint32_t b0 = 0; b0 < B && e == cudaSuccess; b0 += kPlainMaxB) {
@@ -393,13 +393,13 @@ tpir_status enqueue_multi(const tpir_read_job* jobs, uint32_t njobs, cudaStream_
     if (kind == 4) {
       (q.B > 256 ? m4w : m4).push_back(r);
     } else if (kind == 5) {
+      if (!tensor_mid(q.db, q.B) || q.db->forced_kernel) q.db->tt_wanted = true;
       const cudaError_t e = tcopy_ensure(q.db, st);
       if (e == cudaErrorMemoryAllocation && q.db->forced_kernel == 0) {
         lop3.push_back(q);  // no room for the copy
         continue;
       }
       if (e != cudaSuccess) return cuda_status(e);
-      if (!tensor_mid(q.db, q.B)) q.db->tt_wanted = true;
       M4Request t = r;
       t.Tt = q.db->d_tt;
       tc.push_back(t);
@@ -890,9 +890,9 @@ tpir_status tpir_read_multi_graph_create(const tpir_read_job* jobs, uint32_t njo
     tpir_db* db = jobs[i].db;
     order_writes_after_reads(db, db->stream);
     cudaError_t e = cudaStreamWaitEvent(db->stream, db->last_write, 0);
+    db->tt_wanted = true;  // replays read the copy as it then is
     if (e == cudaSuccess) e = tcopy_ensure(db, db->stream);
     if (e == cudaErrorMemoryAllocation && db->forced_kernel == 0) continue;  // read by another kernel
-    db->tt_wanted = true;  // replays read the copy as it then is
     if (e == cudaSuccess) e = cudaEventRecord(db->last_write, db->stream);
     if (e != cudaSuccess) {
       delete g;

@@ -183,6 +183,7 @@ tpir_status tpir_autotune(tpir_db* db, uint32_t B, uint32_t reps, tpir_tune_resu
   double best_k_us = best;
   double us_tensor = 0.0, us_m4rm = 0.0, us_plain = 0.0;
   uint32_t tensor_tried = 0;
+  if (B > kPlainMaxB) db->tt_wanted = true;
   if (e == cudaSuccess && tcopy_ensure(db, st) == cudaSuccess) {  // (no room for the copy: not tried)
     std::vector<GSched> scheds;
     // mode 1 (table operand in tensor memory) and, above 128 requests, mode 2

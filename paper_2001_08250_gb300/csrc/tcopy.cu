@@ -100,7 +100,16 @@ uint64_t tcopy_bytes(uint64_t n, uint32_t row_bytes) { return (n + 63) / 64 * 64
 cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
   if (db->tt_valid) return cudaSuccess;
   if (!db->d_tt) {
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&db->d_tt), tcopy_bytes(db->n, db->row_bytes));
+    const uint64_t bytes = tcopy_bytes(db->n, db->row_bytes);
+    if (!db->tt_wanted) {  // only for the smaller batches: not if it would make memory scarce
+      size_t free_b = 0, total_b = 0;
+      if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || bytes > free_b / 4) {
+        cudaGetLastError();
+        db->tt_denied = true;
+        return cudaErrorMemoryAllocation;
+      }
+    }
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&db->d_tt), bytes);
     if (e != cudaSuccess) {
       db->d_tt = nullptr;
       db->tt_denied = e == cudaErrorMemoryAllocation;

@@ -11,8 +11,8 @@
 //                        buckets past n are zero.
 //
 // The copy is built in full on first use and after a bulk load, and block by
-// block after the slot moves of a write (only the 64-bucket blocks holding a
-// moved slot), in the same stream order as the table itself, so it always
+// block after the slot moves of a write (only the moved slots' columns of the
+// 64-bucket blocks holding them), in the same stream order as the table itself, so it always
 // matches the table for every later read.
 #include <algorithm>
 #include <vector>
@@ -31,27 +31,30 @@ namespace {
 // over the 64 buckets (32 lanes x 8 bytes stored, contiguous).
 // Bound by HBM: a load of 32 768 x 4 KiB takes 74 us for its three passes over
 // 128 MiB (312 and a copy of 40 before it when each warp read 32 rows' words 4 KiB
-// apart and took 64 ballots a word); 256 blocks after a batch of writes 21 (126).
+// apart and took 64 ballots a word); the columns of the slots that 256 writes
+// touched 8.42 (126 then and 21 now by whole rows).
 template <bool COPY>
 __global__ void __launch_bounds__(256) tcopy_kernel(const uint4* __restrict__ src, uint64_t n, uint32_t Wd,
                                                     uint4* __restrict__ table, uint64_t* __restrict__ Tt,
                                                     uint64_t nblocks, const __grid_constant__ TcopyBlocks bl) {
   __shared__ uint32_t tile[64][33];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t chunks = (Wd + 31) / 32, U = Wd / 4;
+  const uint32_t Ws = bl.count ? bl.slot_words : Wd;  // words of an entry: a slot, or the row
+  const uint32_t chunks = (Ws + 31) / 32, U = Wd / 4;
   const uint64_t items = (bl.count ? bl.count : nblocks) * chunks;
   const uint64_t row_bits = static_cast<uint64_t>(Wd) * 32;
   const WarpTranspose transpose;
   for (uint64_t it = blockIdx.x; it < items; it += gridDim.x) {
     const uint64_t kb = bl.count ? bl.kb[it / chunks] : it / chunks;
-    const uint32_t w0 = static_cast<uint32_t>(it % chunks) * 32;
+    const uint32_t wb = bl.count ? bl.slot[it / chunks] * Ws : 0u;  // first word, and past the last
+    const uint32_t w0 = wb + static_cast<uint32_t>(it % chunks) * 32, we = wb + Ws;
     // thread: 16 bytes of rows threadIdx / 8 and 32 + threadIdx / 8
     const uint32_t r = threadIdx.x >> 3, u = threadIdx.x & 7u, uc = w0 / 4 + u;
     uint4 v[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
 #pragma unroll
     for (uint32_t h = 0; h < 2; ++h) {
       const uint64_t row = 64 * kb + 32 * h + r;
-      if (row < n && uc < U) v[h] = src[row * U + uc];
+      if (row < n && 4 * uc < we) v[h] = src[row * U + uc];
     }
     __syncthreads();  // the tile's last readers are done
 #pragma unroll
@@ -68,7 +71,7 @@ __global__ void __launch_bounds__(256) tcopy_kernel(const uint4* __restrict__ sr
 #pragma unroll
     for (uint32_t i = 0; i < 4; ++i) {
       const uint32_t c = 4 * warp + i;
-      if (w0 + c >= Wd) break;  // uniform over the warp
+      if (w0 + c >= we) break;  // uniform over the warp
       const uint32_t lo = transpose(tile[lane][c]), hi = transpose(tile[32 + lane][c]);
       Tt[kb * row_bits + static_cast<uint64_t>(w0 + c) * 32 + lane] =
           static_cast<uint64_t>(lo) | (static_cast<uint64_t>(hi) << 32);
@@ -79,7 +82,8 @@ __global__ void __launch_bounds__(256) tcopy_kernel(const uint4* __restrict__ sr
 // src: the table itself, or (all blocks) device memory to copy to it as well
 cudaError_t launch_tcopy(const tpir_db* db, const void* src, const TcopyBlocks& bl, cudaStream_t st) {
   const uint64_t nblocks = (db->n + 63) / 64;
-  const uint64_t items = (bl.count ? bl.count : nblocks) * ((db->Wd + 31) / 32);
+  const uint64_t items = bl.count ? static_cast<uint64_t>(bl.count) * ((bl.slot_words + 31) / 32)
+                                  : nblocks * ((db->Wd + 31) / 32);
   if (items == 0) return cudaSuccess;
   const uint32_t grid = static_cast<uint32_t>(
       std::min<uint64_t>(items, static_cast<uint64_t>(device_sm_count()) * 8));
@@ -164,7 +168,8 @@ cudaError_t tcopy_after_moves(tpir_db* db, const MoveOp* ops, size_t nops, cudaS
   std::vector<uint64_t> kbs;
   kbs.reserve(nops);
   for (size_t i = 0; i < nops; ++i)
-    if (ops[i].dst != kTmpSlot) kbs.push_back(ops[i].dst / db->d / 64);
+    if (ops[i].dst != kTmpSlot)  // (block, slot of the bucket)
+      kbs.push_back(ops[i].dst / db->d / 64 * db->d + ops[i].dst % db->d);
   std::sort(kbs.begin(), kbs.end());
   kbs.erase(std::unique(kbs.begin(), kbs.end()), kbs.end());
   if (!db->tt_wanted && kbs.size() > 16) {  // as after a load
@@ -172,9 +177,20 @@ cudaError_t tcopy_after_moves(tpir_db* db, const MoveOp* ops, size_t nops, cudaS
     db->mid_reads = 0;
     return cudaSuccess;
   }
+  uint32_t d = db->d;
+  bl.slot_words = db->z / 4;
+  if (kbs.size() > kTcopyMaxBlocks) {  // too many slots to list: their blocks, by whole rows
+    for (uint64_t& k : kbs) k /= d;
+    kbs.erase(std::unique(kbs.begin(), kbs.end()), kbs.end());
+    d = 1;
+    bl.slot_words = db->Wd;
+  }
   if (kbs.size() > kTcopyMaxBlocks) return launch_tcopy(db, db->d_table, bl, st);  // rebuild it all
   bl.count = static_cast<uint32_t>(kbs.size());
-  std::copy(kbs.begin(), kbs.end(), bl.kb);
+  for (size_t i = 0; i < kbs.size(); ++i) {
+    bl.kb[i] = kbs[i] / d;
+    bl.slot[i] = static_cast<uint8_t>(kbs[i] % d);
+  }
   return launch_tcopy(db, db->d_table, bl, st);
 }
 

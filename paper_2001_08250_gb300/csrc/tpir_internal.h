@@ -218,9 +218,10 @@ cudaError_t launch_bloom_union(const uint64_t* deltas, uint32_t window, uint64_t
 // Tt[kb][c] holds bit c of the rows of buckets 64 kb .. 64 kb + 63.
 constexpr uint32_t kTcopyMaxBlocks = 480;  // blocks a partial rebuild takes by value
 struct TcopyBlocks {
-  uint32_t count;  // 0: every block
-  uint32_t pad;
+  uint32_t count;       // entries (a slot of the buckets of a block each); 0: every block, whole rows
+  uint32_t slot_words;  // words of a slot
   uint64_t kb[kTcopyMaxBlocks];
+  uint8_t slot[kTcopyMaxBlocks];
 };
 static_assert(sizeof(TcopyBlocks) + 64 < 32000, "kernel parameters must stay below 32 KB");
 uint64_t tcopy_bytes(uint64_t n, uint32_t row_bytes);

@@ -161,6 +161,7 @@ int auto_kernel(const tpir_db* db, uint32_t B) {
 // HBM at a higher rate.
 bool tensor_mid(const tpir_db* db, uint32_t B) {
   if (B <= kPlainMaxB || (B >= kTensorMinB && db->Wd >= kTensorMinWd)) return false;
+  if (db->row_bytes > (1u << 27)) return false;  // (the copy's tensor map counts columns in 32 bits)
   return B > 8 || db->row_bytes < 2048 || db->n * db->row_bytes <= (96ull << 20);
 }
 

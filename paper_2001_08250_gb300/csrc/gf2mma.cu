@@ -739,7 +739,7 @@ int p_max_pairs() {
 
 // Clocks of the pair form on the whole device, launch included, and its
 // k-chunk rows (rounds x item time, about 119 cycles per pair MMA, two per
-// K-step; the measured launches took 1.15 times that and 7 us: 85 us for 64 at
+// K-step; the measured launches took 1.21 times that and 5 us: 83 us for 64 at
 // 256 requests of 32 768 x 4 KiB, 10.8 for 3.5 at 1 024 x 4 KiB).
 double g_pair_plan(uint64_t n, uint32_t Wd, uint32_t B, int pairs, uint32_t* kc_rows) {
   const GJob J = g_job(nullptr, 0, B, nullptr, nullptr, n, Wd);
@@ -760,7 +760,7 @@ double g_pair_plan(uint64_t n, uint32_t Wd, uint32_t B, int pairs, uint32_t* kc_
       *kc_rows = static_cast<uint32_t>(rows);
     }
   }
-  return 1.15 * best + 13000.0;
+  return 1.21 * best + 10000.0;
 }
 
 // One job on CTA pairs (B > 128, request rows TMA-staged): items of whole

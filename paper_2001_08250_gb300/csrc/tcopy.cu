@@ -32,7 +32,7 @@ namespace {
 // Bound by HBM: a load of 32 768 x 4 KiB takes 74 us for its three passes over
 // 128 MiB (312 and a copy of 40 before it when each warp read 32 rows' words 4 KiB
 // apart and took 64 ballots a word); the columns of the slots that 256 writes
-// touched 8.42 (126 then and 21 now by whole rows).
+// touched 8.4 (126 then and 21 now by whole rows).
 template <bool COPY>
 __global__ void __launch_bounds__(256) tcopy_kernel(const uint4* __restrict__ src, uint64_t n, uint32_t Wd,
                                                     uint4* __restrict__ table, uint64_t* __restrict__ Tt,

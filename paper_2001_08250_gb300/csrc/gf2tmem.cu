@@ -120,7 +120,8 @@ struct TJob {
   uint32_t kcs, kc_words;
   uint32_t splits;       // column tiles t, t + splits, ... form one item
   uint32_t item_begin;
-  uint32_t split;        // 0: replies stored; 1: initialised first, XOR-reduced into
+  uint32_t split;        // 0: replies stored; 1: initialised first (zeros or masks), XOR-reduced
+                         // into; 2: masked, stored by their single writer with the mask
 };
 
 template <int NJ>
@@ -324,6 +325,23 @@ __device__ __forceinline__ void t_load_requests(const TJob& J, const TItem& it, 
       }
     }
   }
+}
+
+// Words w and w + 1 (w even) of the mask with this seed: words w % 16 and the next
+// of ChaCha20 block w / 16, by selects (an index not known at compile time would
+// send the block to local memory).
+__device__ __noinline__ uint64_t t_mask(const uint8_t* seed, uint32_t w) {
+  const uint4 ka = __ldg(reinterpret_cast<const uint4*>(seed)), kb = __ldg(reinterpret_cast<const uint4*>(seed) + 1);
+  const uint32_t key[8] = {ka.x, ka.y, ka.z, ka.w, kb.x, kb.y, kb.z, kb.w};
+  uint32_t k[16];
+  cc_block(key, w >> 4, k);
+  uint32_t lo = k[0], hi = k[1];
+#pragma unroll
+  for (uint32_t i = 2; i < 16; i += 2) {
+    lo = (w & 15u) == i ? k[i] : lo;
+    hi = (w & 15u) == i ? k[i + 1] : hi;
+  }
+  return lo | static_cast<uint64_t>(hi) << 32;
 }
 
 template <int NJ, int G>
@@ -660,8 +678,10 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
         if (q < N && b < J.B) {
           uint64_t v;
           asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(ob + et * 8u) : "memory");
-          uint32_t* p = J.out + static_cast<uint64_t>(b) * J.Wd + t * 4u + (et & 1u) * 2u;
-          if (J.split)
+          const uint32_t w = t * 4u + (et & 1u) * 2u;
+          uint32_t* p = J.out + static_cast<uint64_t>(b) * J.Wd + w;
+          if (J.split == 2) v ^= t_mask(J.seeds + static_cast<uint64_t>(b) * 32, w);
+          if (J.split == 1)
             asm volatile("red.relaxed.gpu.global.xor.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
           else
             *reinterpret_cast<uint64_t*>(p) = v;
@@ -730,7 +750,12 @@ void t_set_chunks(TJob& j, uint32_t kc_words, uint32_t splits) {
   j.kc_words = kc_words;
   j.kcs = (j.nw + kc_words - 1) / kc_words;
   j.splits = splits;
-  j.split = (j.kcs > 1 || j.seeds) ? 1u : 0u;
+  // a masked read of a table so small that every CTA has a tile at most forms
+  // the masks where it stores (a keystream block per eight bytes, but no launch
+  // before it: 90 masked reads of 1 132 x 256 bytes 5.4 us, 6.8 with one); larger
+  // ones have them written first, a block per 64 bytes
+  const bool small = static_cast<uint64_t>(j.mbs) * j.tiles <= static_cast<uint64_t>(device_sm_count());
+  j.split = j.kcs > 1 ? 1u : !j.seeds ? 0u : small ? 2u : 1u;
 }
 
 uint32_t t_min_chunks(const TJob& j) {
@@ -753,7 +778,9 @@ double t_plan(TJob& j, uint32_t grid) {
       const uint32_t st = (j.tiles + s - 1) / s;
       const uint64_t items = per * s;
       const uint64_t rounds = (items + grid - 1) / grid;
-      const double cost = static_cast<double>(rounds) * t_item_clk(j.mb_rows, kw, st);
+      // (the replies' initialisation, a launch, costs a read of several k-chunks
+      // 3 000 clocks: a small table is read in one)
+      const double cost = static_cast<double>(rounds) * t_item_clk(j.mb_rows, kw, st) + (kw < j.nw ? 3000.0 : 0.0);
       if (cost < best) {
         best = cost;
         bw = kw;
@@ -800,7 +827,7 @@ cudaError_t t_scan(TLaunch<NJ>& L, cudaStream_t st) {
 double gf2_tmem_clk(uint64_t n, uint32_t Wd, uint32_t B, bool masked) {
   TJob j = t_job(nullptr, 0, B, nullptr, nullptr, n, Wd);
   const double clk = t_plan(j, static_cast<uint32_t>(device_sm_count()));
-  return 1.04 * (clk + (j.split || masked ? 4000.0 : 1000.0));
+  return 1.04 * (clk + (masked && j.kcs == 1 ? 4000.0 : 1000.0));
 }
 
 cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const uint64_t* R,

@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
   __shared__ __align__(8) uint64_t full[kTStreams][kTSlots], empty[kTStreams][kTSlots];
   __shared__ __align__(8) uint64_t raw_full[kTStreams][kTRaw], raw_empty[kTStreams][kTRaw];
   __shared__ __align__(8) uint64_t accf[kTStreams][2], acce[kTStreams][2], drain[kTStreams];
-  __shared__ __align__(8) uint64_t reqf, outf;
+  __shared__ __align__(8) uint64_t reqf, reqe, outf;
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
   uint8_t* base = reinterpret_cast<uint8_t*>(
@@ -381,6 +381,7 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
       }
     }
     mb::init(&reqf, kTEpiWarps);
+    mb::init(&reqe, kTStreams);
     mb::init(&outf, kTEpiWarps);
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -478,6 +479,9 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
       const uint32_t idesc = (1u << 7) | (1u << 10) | ((N >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24);
       const uint32_t dstep = (32u * N) >> 4;
       if (!t_wait_warp(&reqf, r & 1u, abort_flag, status)) break;
+      // (an issuer without a tile in this item says so too: the next phase of
+      // reqf completes only after both have seen this one)
+      if (one) mb::arrive(&reqe);
       const uint32_t W = it.w1 - it.w0;
       for (uint32_t i = g; ok && i < it.nt; i += kTStreams, ++tc) {
         const uint32_t buf = nb2 & tc, acc = utmem + g * kTAcc + buf * kTAccHalf;
@@ -650,10 +654,11 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
         if (more && i + 1 == it.nt) {
           // every tile's MMAs have read the item's requests: the next item's
           // go in before this tile's replies, so that its MMAs start the sooner
+          // (and are announced once both issuers have seen this item's)
           t_load_requests(L.jobs[nx.job], nx, res0, warp - kTEpiWarp0, lane);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
-          if (lane == 0) mb::arrive(&reqf);
+          if (lane == 0 && mb::wait(&reqe, r & 1u, abort_flag, status, kTWaitNs)) mb::arrive(&reqf);
         }
         const WarpTranspose transpose;  // formed anew for each tile: its registers are the counts' before
         const uint32_t ob = out0 + (te & 1u) * kTOutBytes, oq = ob + (c0 + lane) * 16u + quarter * 4u;

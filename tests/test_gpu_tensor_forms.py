@@ -83,3 +83,35 @@ def test_smaller_batches_before_and_after_the_transposed_copy(n, d, z, B):
         assert np.array_equal(to_host(job[3]), exp)
         g.close()
     assert talekpir.device_status() == talekpir.OK
+
+
+@pytest.mark.parametrize("n,d,z,B", [(200003, 1, 16, 1024), (200003, 1, 16, 784), (120001, 3, 16, 784),
+                                     (90001, 1, 16, 769)])
+def test_items_of_one_tile_one_after_another(n, d, z, B):
+    """Narrow rows with many request blocks and k-chunks: a CTA takes several items
+    of one column tile (or of three, one stream with a tile more), in which the
+    second stream has none; alone and with another table of such items."""
+    require_cuda()
+    T = synth.table_bytes(n, d, z, seed=180, table=n)
+    R = synth.random_bits(B, n, seed=181, table=n)
+    exp = oracle.read_batch(T, n, d, z, R)
+    n2, B2 = 70001, 900
+    T2 = synth.table_bytes(n2, 1, 48, seed=182, table=n2)
+    R2 = synth.random_bits(B2, n2, seed=183, table=n2)
+    exp2 = oracle.read_batch(T2, n2, 1, 48, R2)
+    with talekpir.DB(n, d, z) as db, talekpir.DB(n2, 1, 48) as db2:
+        db.load(T)
+        db2.load(T2)
+        dR, dR2 = to_dev(R), to_dev(R2)
+        for x in (db, db2):
+            x.set_kernel(TENSOR)
+        outs = [dev_out(B, d * z) for _ in range(12)]
+        for out in outs:
+            db.read_batch_async(dR, B, out)
+        for out in outs:
+            assert np.array_equal(to_host(out), exp)
+        out, out2 = dev_out(B, d * z), dev_out(B2, 48)
+        for _ in range(4):
+            talekpir.read_multi_async([(db, B, dR, out), (db2, B2, dR2, out2)])
+        assert np.array_equal(to_host(out), exp) and np.array_equal(to_host(out2), exp2)
+    assert talekpir.device_status() == talekpir.OK

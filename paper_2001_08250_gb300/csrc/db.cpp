@@ -148,7 +148,8 @@ int auto_kernel(const tpir_db* db, uint32_t B) {
   // runs on the register-tiled kernel, so that a table read once does not pay
   // for the copy
   if (B <= kPlainMaxB) return 1;
-  if (tensor_mid(db, B)) return !db->tt_denied && (db->tt_valid || db->mid_reads) ? 5 : 2;
+  if (tensor_mid(db, B))
+    return db->tt_valid || (db->mid_reads && !db->tt_denied && !db->tt_scarce) ? 5 : 2;
   return B >= kTensorMinB && db->Wd >= kTensorMinWd && !db->tt_denied ? 5 : 2;
 }
 

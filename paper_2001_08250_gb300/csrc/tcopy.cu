@@ -109,7 +109,7 @@ cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
       size_t free_b = 0, total_b = 0;
       if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || bytes > free_b / 4) {
         cudaGetLastError();
-        db->tt_denied = true;
+        db->tt_scarce = true;
         return cudaErrorMemoryAllocation;
       }
     }
@@ -144,7 +144,7 @@ bool tcopy_load(tpir_db* db, const void* src, cudaStream_t st, cudaError_t* e) {
   const uint64_t bytes = db->n * db->row_bytes;
   if (s8 < db->d_table + bytes && db->d_table < s8 + bytes) return false;  // overlapping: a plain copy
   TcopyBlocks all{};
-  db->tt_denied = false;
+  db->tt_denied = db->tt_scarce = false;
   db->tt_valid = false;
   *e = launch_tcopy(db, src, all, st);
   if (*e == cudaSuccess) db->tt_valid = true;
@@ -152,7 +152,7 @@ bool tcopy_load(tpir_db* db, const void* src, cudaStream_t st, cudaError_t* e) {
 }
 
 cudaError_t tcopy_after_load(tpir_db* db, cudaStream_t st) {
-  db->tt_denied = false;
+  db->tt_denied = db->tt_scarce = false;
   if (!db->d_tt) return cudaSuccess;  // built on first use
   db->tt_valid = false;
   if (!db->tt_wanted) {  // only smaller batches used it: made again by the second of them

@@ -391,6 +391,8 @@ struct tpir_db {
   bool tt_wanted = false;  // large batches, tuned or forced reads or a captured graph use it: kept
                            // equal to the table at every load and write
   bool tt_denied = false;  // there was no room for it; asked for again after a load
+  bool tt_scarce = false;  // refused to a smaller batch, as it would have made memory scarce (a
+                           // large one still asks for it); until a load
   uint32_t mid_reads = 0;  // 1: a batch of tensor_mid size was read without the copy
 };
 

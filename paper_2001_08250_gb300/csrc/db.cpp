@@ -138,10 +138,15 @@ uint32_t next_counter_slot() {
   return next.fetch_add(1, std::memory_order_relaxed) % kItemCounterSlots;
 }
 
-int auto_kernel(const tpir_db* db, uint32_t B) {
+int told_kernel(const tpir_db* db, uint32_t B) {
   if (db->forced_kernel) return db->forced_kernel;
   KernelPlan kp;
-  if (kernel_plan_lookup(db->Wd, B, db->n, &kp)) return kp.kernel;  // measured winner
+  if (!kernel_plan_lookup(db->Wd, B, db->n, &kp)) return 0;
+  return kp.kernel == 5 && db->tt_denied ? 2 : kp.kernel;  // (no room for its copy)
+}
+
+int auto_kernel(const tpir_db* db, uint32_t B) {
+  if (const int told = told_kernel(db, B)) return told;
   // plain stream for a few requests; the tensor-core kernel for large batches
   // on wide rows, and for the others it is faster at (tensor_mid) once the
   // table has its transposed copy, or had one such batch before: the first
@@ -361,9 +366,8 @@ int multi_kernel(const tpir_read_job& q) {
   if (forced == 4 && q.db->Wd >= 64) return 4;
   if (forced == 5) return 5;
   if (forced == 0) {
-    KernelPlan kp;
-    if (kernel_plan_lookup(q.db->Wd, q.B, q.db->n, &kp)) {
-      if (kp.kernel == 5 || (kp.kernel == 4 && q.db->Wd >= 64)) return kp.kernel;
+    if (const int told = told_kernel(q.db, q.B)) {
+      if (told == 5 || (told == 4 && q.db->Wd >= 64)) return told;
       return 2;  // the plain kernel's jobs run in the register-tiled launch
     }
     if (q.db->tt_denied) return 2;

@@ -416,7 +416,11 @@ tpir_status cuda_status(cudaError_t e);
 tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d_out,
                          cudaStream_t st, const uint8_t* d_seeds = nullptr,
                          int* kernel_used = nullptr, int kernel_choice = 0);
-// The kernel a read of B requests takes on db unless told otherwise.
+// The kernel a read of B requests is told to take on db: a forced one, or a tuned
+// plan's (register-tiled in place of a tensor-core one whose copy was refused);
+// 0: none.
+int told_kernel(const tpir_db* db, uint32_t B);
+// The kernel it takes.
 int auto_kernel(const tpir_db* db, uint32_t B);
 // A batch, other than the large ones on wide rows, that the tensor-core kernel
 // reads faster than the register-tiled one.

@@ -68,3 +68,35 @@ def test_a_refusal_for_small_batches_leaves_large_ones_their_copy():
         torch.cuda.empty_cache()
         t.db.close()
     assert talekpir.device_status() == talekpir.OK
+
+
+def test_a_tuned_tensor_kernel_without_room_for_its_copy(tmp_path):
+    """Reads, many-table calls and captured graphs run on the register-tiled kernel,
+    and the refused copy is not asked for by each of them."""
+    torch = require_cuda()
+    t = Table()
+    plan = tmp_path / "plan.json"
+    plan.write_text('{"plans": [\n' + "".join(
+        '{"row_words": %d, "batch_class": %d, "n_class": 10, "kernel": 5, "tensor_mode": 1, '
+        '"tensor_kc_rows": 0, "tensor_loads": 0}\n' % (ROW // 4, c) for c in (4, 6)) + "]}\n")
+    talekpir.tune_load(str(plan))
+    x = fill(torch, 160 << 20)
+    try:
+        for B in (LARGE, MID):
+            job = (t.db, B, t.R, t.out)
+            t.out.zero_()
+            g = talekpir.MultiGraph([job])
+            g.launch()
+            torch.cuda.synchronize()
+            assert (t.out[:B] == t.expected[:B]).all()
+            g.close()
+            assert t.read(B) == 2
+            t.out.zero_()
+            talekpir.read_multi_async([job])
+            assert (t.out[:B] == t.expected[:B]).all()
+    finally:
+        talekpir.tune_clear()
+        del x
+        torch.cuda.empty_cache()
+        t.db.close()
+    assert talekpir.device_status() == talekpir.OK

@@ -180,7 +180,7 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
   const int kernel = kernel_choice ? kernel_choice : auto_kernel(db, B);
   if (kernel_used) *kernel_used = kernel;
   cudaError_t e = cudaSuccess;
-  if (kernel == 5 && (!tensor_mid(db, B) || db->forced_kernel)) db->tt_wanted = true;
+  if (kernel == 5 && (!tensor_mid(db, B) || told_kernel(db, B) == 5)) db->tt_wanted = true;
   if (kernel == 5 && kernel_choice == 0 && db->forced_kernel == 0) {
     // no room for the copy: the register-tiled kernel
     e = tcopy_ensure(db, st);
@@ -399,7 +399,7 @@ tpir_status enqueue_multi(const tpir_read_job* jobs, uint32_t njobs, cudaStream_
     if (kind == 4) {
       (q.B > 256 ? m4w : m4).push_back(r);
     } else if (kind == 5) {
-      if (!tensor_mid(q.db, q.B) || q.db->forced_kernel) q.db->tt_wanted = true;
+      if (!tensor_mid(q.db, q.B) || told_kernel(q.db, q.B) == 5) q.db->tt_wanted = true;
       const cudaError_t e = tcopy_ensure(q.db, st);
       if (e == cudaErrorMemoryAllocation && q.db->forced_kernel == 0) {
         lop3.push_back(q);  // no room for the copy

@@ -100,3 +100,26 @@ def test_a_tuned_tensor_kernel_without_room_for_its_copy(tmp_path):
         torch.cuda.empty_cache()
         t.db.close()
     assert talekpir.device_status() == talekpir.OK
+
+
+def test_a_tuned_small_batch_has_its_copy_as_a_large_one(tmp_path):
+    """A plan that names the tensor-core kernel for a small batch asks for the copy:
+    it is made at the first read, and kept at a load."""
+    torch = require_cuda()
+    t = Table()
+    plan = tmp_path / "plan.json"
+    plan.write_text('{"plans": [\n{"row_words": %d, "batch_class": 4, "n_class": 10, "kernel": 5, '
+                    '"tensor_mode": 1, "tensor_kc_rows": 0, "tensor_loads": 0}\n]}\n' % (ROW // 4))
+    table = torch.as_tensor(t.db.dump()).cuda()
+    talekpir.tune_load(str(plan))
+    x = fill(torch, 640 << 20)
+    try:
+        assert [t.read(MID) for _ in range(2)] == [2, 1]  # copy and scan, scan
+        t.db.load_async(table)
+        assert t.read(MID) == 1
+    finally:
+        talekpir.tune_clear()
+        del x
+        torch.cuda.empty_cache()
+        t.db.close()
+    assert talekpir.device_status() == talekpir.OK

@@ -142,7 +142,7 @@ int told_kernel(const tpir_db* db, uint32_t B) {
   if (db->forced_kernel) return db->forced_kernel;
   KernelPlan kp;
   if (!kernel_plan_lookup(db->Wd, B, db->n, &kp)) return 0;
-  return kp.kernel == 5 && db->tt_denied ? 2 : kp.kernel;  // (no room for its copy)
+  return kp.kernel == 5 && db->tt_skip ? 2 : kp.kernel;  // (no room for its copy)
 }
 
 int auto_kernel(const tpir_db* db, uint32_t B) {
@@ -154,8 +154,8 @@ int auto_kernel(const tpir_db* db, uint32_t B) {
   // for the copy
   if (B <= kPlainMaxB) return 1;
   if (tensor_mid(db, B))
-    return db->tt_valid || (db->mid_reads && !db->tt_denied && !db->tt_scarce) ? 5 : 2;
-  return B >= kTensorMinB && db->Wd >= kTensorMinWd && !db->tt_denied ? 5 : 2;
+    return db->tt_valid || (db->mid_reads && !db->tt_skip && !db->tt_scarce) ? 5 : 2;
+  return B >= kTensorMinB && db->Wd >= kTensorMinWd && !db->tt_skip ? 5 : 2;
 }
 
 // Batches other than the large ones on wide rows that the tensor-core kernel
@@ -177,6 +177,7 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
   if (B == 0) return TPIR_OK;
   d_req += db->req_off;  // a row shard reads its own words of each request row
   order_after_writes(db, st);
+  if (kernel_choice == 0 && db->tt_skip) --db->tt_skip;
   const int kernel = kernel_choice ? kernel_choice : auto_kernel(db, B);
   if (kernel_used) *kernel_used = kernel;
   cudaError_t e = cudaSuccess;
@@ -370,7 +371,7 @@ int multi_kernel(const tpir_read_job& q) {
       if (told == 5 || (told == 4 && q.db->Wd >= 64)) return told;
       return 2;  // the plain kernel's jobs run in the register-tiled launch
     }
-    if (q.db->tt_denied) return 2;
+    if (q.db->tt_skip) return 2;
     if (q.B >= kTensorMinB && q.db->Wd >= kTensorMinWd) return 5;
     if (tensor_mid(q.db, q.B) && q.db->tt_valid) return 5;
   }
@@ -865,7 +866,10 @@ tpir_status tpir_read_multi_async(const tpir_read_job* jobs, uint32_t njobs, voi
   for (uint32_t i = 0; i < njobs; ++i)
     if (!jobs[i].db) return TPIR_EINVAL;
   for (uint32_t i = 0; i < njobs; ++i)
-    if (jobs[i].B) order_after_writes(jobs[i].db, st);
+    if (jobs[i].B) {
+      order_after_writes(jobs[i].db, st);
+      if (jobs[i].db->tt_skip) --jobs[i].db->tt_skip;
+    }
   tpir_status s = enqueue_multi(jobs, njobs, st);
   if (s != TPIR_OK) return s;
   for (uint32_t i = 0; i < njobs; ++i)

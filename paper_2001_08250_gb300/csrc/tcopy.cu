@@ -116,10 +116,12 @@ cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&db->d_tt), bytes);
     if (e != cudaSuccess) {
       db->d_tt = nullptr;
-      db->tt_denied = e == cudaErrorMemoryAllocation;
+      if (e == cudaErrorMemoryAllocation) db->tt_skip = kTcopySkip;
       cudaGetLastError();
       return e;
     }
+    db->tt_skip = 0;
+    db->tt_scarce = false;
   }
   TcopyBlocks all{};
   cudaError_t e = launch_tcopy(db, db->d_table, all, st);
@@ -144,7 +146,8 @@ bool tcopy_load(tpir_db* db, const void* src, cudaStream_t st, cudaError_t* e) {
   const uint64_t bytes = db->n * db->row_bytes;
   if (s8 < db->d_table + bytes && db->d_table < s8 + bytes) return false;  // overlapping: a plain copy
   TcopyBlocks all{};
-  db->tt_denied = db->tt_scarce = false;
+  db->tt_skip = 0;
+  db->tt_scarce = false;
   db->tt_valid = false;
   *e = launch_tcopy(db, src, all, st);
   if (*e == cudaSuccess) db->tt_valid = true;
@@ -152,7 +155,8 @@ bool tcopy_load(tpir_db* db, const void* src, cudaStream_t st, cudaError_t* e) {
 }
 
 cudaError_t tcopy_after_load(tpir_db* db, cudaStream_t st) {
-  db->tt_denied = db->tt_scarce = false;
+  db->tt_skip = 0;
+  db->tt_scarce = false;
   if (!db->d_tt) return cudaSuccess;  // built on first use
   db->tt_valid = false;
   if (!db->tt_wanted) {  // only smaller batches used it: made again by the second of them

@@ -216,6 +216,10 @@ cudaError_t launch_bloom_union(const uint64_t* deltas, uint32_t window, uint64_t
 
 // Bit-transposed copy of a table for the tensor-core read (tcopy.cu):
 // Tt[kb][c] holds bit c of the rows of buckets 64 kb .. 64 kb + 63.
+// Reads that do without a copy for which there was no room before it is asked for
+// again: by then others may have given memory back, and a refused allocation is
+// spread over so many reads.
+constexpr uint32_t kTcopySkip = 256;
 constexpr uint32_t kTcopyMaxBlocks = 480;  // blocks a partial rebuild takes by value
 struct TcopyBlocks {
   uint32_t count;       // entries (a slot of the buckets of a block each); 0: every block, whole rows
@@ -390,7 +394,8 @@ struct tpir_db {
   bool tt_valid = false;
   bool tt_wanted = false;  // large batches, tuned or forced reads or a captured graph use it: kept
                            // equal to the table at every load and write
-  bool tt_denied = false;  // there was no room for it; asked for again after a load
+  uint32_t tt_skip = 0;    // there was no room for it: so many reads do without before it is asked
+                           // for again (0 after a load)
   bool tt_scarce = false;  // refused to a smaller batch, as it would have made memory scarce (a
                            // large one still asks for it); until a load
   uint32_t mid_reads = 0;  // 1: a batch of tensor_mid size was read without the copy

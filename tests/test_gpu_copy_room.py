@@ -123,3 +123,24 @@ def test_a_tuned_small_batch_has_its_copy_as_a_large_one(tmp_path):
         torch.cuda.empty_cache()
         t.db.close()
     assert talekpir.device_status() == talekpir.OK
+
+
+def test_a_copy_there_was_no_room_for_is_asked_for_again():
+    """Once memory has been given back, a table whose copy was refused gets it, by
+    single reads as by many-table calls, without a load in between."""
+    torch = require_cuda()
+    t = Table()
+    x = fill(torch, 160 << 20)
+    try:
+        assert [t.read(LARGE) for _ in range(3)] == [2] * 3
+        del x
+        torch.cuda.empty_cache()
+        for i in range(300):
+            if i % 2:
+                t.db.read_batch_async(t.R, LARGE, t.out)
+            else:
+                talekpir.read_multi_async([(t.db, LARGE, t.R, t.out)])
+        assert t.read(LARGE) == 1
+    finally:
+        t.db.close()
+    assert talekpir.device_status() == talekpir.OK

@@ -330,12 +330,14 @@ bool form_unit(tpir_server* s, int si, int64_t* next_ready_ns) {
     if (!reads.empty()) {
       // the tensor-core kernel reads a bit-transposed copy of the table (as
       // large as the table), made on first use: only if it fits the budget, and
-      // not for the batches that another kernel reads nearly as well (their
+      // for the smaller batches only if that kernel was forced or tuned (their
       // copies would take the room of tables yet to come)
       int choice = 0;
-      if (tensor_mid(db, B) && !db->d_tt) {
+      if (auto_kernel(db, B) != 5 || db->d_tt) {
+        // nothing to make
+      } else if (tensor_mid(db, B) && told_kernel(db, B) == 0) {
         choice = 2;
-      } else if (auto_kernel(db, B) == 5 && !db->d_tt) {
+      } else {
         const uint64_t tt = tcopy_bytes(db->n, db->row_bytes);
         std::lock_guard<std::mutex> g(s->mu);
         if (s->hbm_tables + s->hbm_tcopies + tt + s->staging_reserve <= s->cfg.hbm_budget_bytes)

@@ -333,6 +333,7 @@ bool form_unit(tpir_server* s, int si, int64_t* next_ready_ns) {
       // for the smaller batches only if that kernel was forced or tuned (their
       // copies would take the room of tables yet to come)
       int choice = 0;
+      uint64_t reserved = 0;
       if (auto_kernel(db, B) != 5 || db->d_tt) {
         // nothing to make
       } else if (tensor_mid(db, B) && told_kernel(db, B) == 0) {
@@ -341,7 +342,7 @@ bool form_unit(tpir_server* s, int si, int64_t* next_ready_ns) {
         const uint64_t tt = tcopy_bytes(db->n, db->row_bytes);
         std::lock_guard<std::mutex> g(s->mu);
         if (s->hbm_tables + s->hbm_tcopies + tt + s->staging_reserve <= s->cfg.hbm_budget_bytes)
-          s->hbm_tcopies += tt;
+          s->hbm_tcopies += reserved = tt;
         else
           choice = 2;
       }
@@ -349,6 +350,10 @@ bool form_unit(tpir_server* s, int si, int64_t* next_ready_ns) {
       cudaMemcpyAsync(sl.d_req, sl.h_req, req_bytes, cudaMemcpyHostToDevice, st);
       const tpir_status r = enqueue_read(db, sl.d_req, B, sl.d_out, st, nullptr, &kernel, choice);
       cudaMemcpyAsync(sl.h_out, sl.d_out, out_bytes, cudaMemcpyDeviceToHost, st);
+      if (reserved && !db->d_tt) {  // there was no room on the device: read without the copy
+        std::lock_guard<std::mutex> g(s->mu);
+        s->hbm_tcopies -= reserved;
+      }
       std::lock_guard<std::mutex> g(s->cmu);
       s->launches++;
       s->batch_tables++;

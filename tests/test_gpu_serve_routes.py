@@ -49,3 +49,32 @@ def test_small_batches_run_on_the_forced_or_tuned_kernel(kernel, tuned, tmp_path
     finally:
         talekpir.tune_clear()
         server.close()
+
+
+def test_a_copy_that_was_not_made_takes_nothing_of_the_budget():
+    """Large batches whose copy the device has no room for, after each of several
+    loads; then a table that the budget holds only without those copies."""
+    torch = require_cuda()
+    n, z, reads = 1000, 65536, 64  # a table of 250 MiB, a copy of 256 MiB
+    server = talekpir.Server(hbm_budget_bytes=(256 + 250 + 256 + 60) << 20, max_inflight=1, tick_us=200000)
+    try:
+        tid = server.add_table(n, D, z)
+        db = server.table(tid)
+        g = torch.Generator(device="cuda")
+        g.manual_seed(230)
+        t = torch.empty(n, D * z // 8, dtype=torch.int64, device="cuda").random_(generator=g)
+        R = synth.random_bits(reads, n, seed=231)
+        out = np.empty((reads, D * z), dtype=np.uint8)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        x = torch.empty(torch.cuda.mem_get_info()[0] - (192 << 20), dtype=torch.uint8, device="cuda")
+        for _ in range(3):
+            db.load_async(t)
+            db.sync()
+            burst(server, tid, R, out)
+        assert server.stats().kernel_launches[2] == 3
+        del x
+        torch.cuda.empty_cache()
+        server.add_table(1000, 4, 100 * 256)  # 98 MiB
+    finally:
+        server.close()

@@ -254,6 +254,8 @@ void CuckooMeta::rollback(const Undo& u) {
 }
 
 std::vector<MoveOp> settle_moves(const std::vector<MoveOp>& ops, uint32_t* nsave) {
+  *nsave = 0;
+  if (ops.size() == 1 && ops[0].kind != 0) return ops;
   // what each slot holds after the moves so far, as a write of it: kind 0 with
   // src = the slot whose original content it is, 1 a payload, 2 zeros
   std::unordered_map<uint64_t, size_t> at;  // slot (or kTmpSlot) -> index in `fin`

@@ -12,29 +12,35 @@
 //  bloom_*_kernel      Section 7: OR a write's interest vector (k positions or
 //                      a whole vector) into the current delta, and form the
 //                      global interest vector as the OR of the window's deltas.
+#include <algorithm>
+
 #include "tpir_internal.h"
 
 namespace tpir {
 namespace {
 
-// Slot writes that do not depend on one another (settle_moves), one CTA each:
-// from a message, a table slot that no write of the list touches, or the saved
-// slots (and the saving itself: kinds 3 and 4), or zeros.
+constexpr uint32_t kMoveThreads = 256;
+
+// Slot writes that do not depend on one another (settle_moves), one column of
+// the grid each: from a message, a table slot that no write of the list touches,
+// or the saved slots (and the saving itself: kinds 3 and 4), or zeros.
 // Bound by latency: 256 writes of 1 KiB take 3.6 us (188 in order in one CTA,
-// 0.7 us a write).
-__global__ void __launch_bounds__(64) settled_moves_kernel(uint8_t* __restrict__ table, uint32_t z,
-                                                           const MoveOp* __restrict__ ops,
-                                                           const uint8_t* __restrict__ payloads,
-                                                           uint8_t* __restrict__ saved) {
+// 0.7 us a write).  A large slot is spread over CTAs: one write of 1 MiB or 16 MiB,
+// the call with its copies to the device, takes 72 and 400 us (150 and 2 250 with 64
+// threads a slot, 111 and 1 270 in order with 256).
+__global__ void __launch_bounds__(kMoveThreads) settled_moves_kernel(uint8_t* __restrict__ table, uint32_t z,
+                                                                     const MoveOp* __restrict__ ops,
+                                                                     const uint8_t* __restrict__ payloads,
+                                                                     uint8_t* __restrict__ saved) {
   const MoveOp op = ops[blockIdx.x];
   uint4* dst = reinterpret_cast<uint4*>(op.kind == 4 ? saved + op.dst * z : table + op.dst * z);
   const uint8_t* s8 = op.kind == 1 ? payloads + op.src * z : op.kind == 3 ? saved + op.src * z : table + op.src * z;
   const uint4* src = reinterpret_cast<const uint4*>(s8);
-  const uint32_t z4 = z / 16;
+  const uint32_t z4 = z / 16, j0 = blockIdx.y * blockDim.x + threadIdx.x, step = gridDim.y * blockDim.x;
   if (op.kind == 2)
-    for (uint32_t j = threadIdx.x; j < z4; j += blockDim.x) dst[j] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t j = j0; j < z4; j += step) dst[j] = make_uint4(0u, 0u, 0u, 0u);
   else
-    for (uint32_t j = threadIdx.x; j < z4; j += blockDim.x) dst[j] = src[j];
+    for (uint32_t j = j0; j < z4; j += step) dst[j] = src[j];
 }
 
 // The ordered moves of a small batch of writes, with the move list and the new
@@ -97,12 +103,15 @@ __global__ void bloom_union_kernel(const uint64_t* __restrict__ deltas, uint32_t
 cudaError_t launch_settled_moves(uint8_t* table, uint32_t z, const MoveOp* ops, uint32_t nsave,
                                  uint32_t nops, const uint8_t* payloads, uint8_t* saved,
                                  cudaStream_t st) {
+  // a thread per 16 bytes of a slot, in up to 1 024 CTAs
+  const uint32_t z4 = z / 16, threads = std::min(kMoveThreads, (z4 + 31) / 32 * 32);
+  const uint32_t y = std::min(1024u, (z4 + threads - 1) / threads);
   if (nsave) {
-    settled_moves_kernel<<<nsave, 64, 0, st>>>(table, z, ops, payloads, saved);
+    settled_moves_kernel<<<dim3(nsave, y), threads, 0, st>>>(table, z, ops, payloads, saved);
     count_launches();
   }
   if (nops > nsave) {
-    settled_moves_kernel<<<nops - nsave, 64, 0, st>>>(table, z, ops + nsave, payloads, saved);
+    settled_moves_kernel<<<dim3(nops - nsave, y), threads, 0, st>>>(table, z, ops + nsave, payloads, saved);
     count_launches();
   }
   return cudaGetLastError();

@@ -217,10 +217,12 @@ tpir_status tpir_xor_combine(const void *const *d_srcs, uint32_t count, uint64_t
                              void *d_dst, void *stream);
 
 /* Force a kernel choice for tests and benchmarks: 0 = automatic (plain for
- * B <= 4, tensor-core for B >= 48 on rows of >= 256 bytes, and from the
- * second such batch of a table for narrower rows and for the smaller batches
- * it is faster at; register-tiled batched otherwise, and where there is no room
- * for the tensor-core kernel's copy of the table), 1 = plain streaming kernel (B <= 4 per launch,
+ * B <= 4, tensor-core for B >= 48 on rows of >= 256 bytes; for narrower rows
+ * and for the smaller batches it is faster at, tensor-core where the table has
+ * that kernel's copy, which such batches earn: it is made for them once they
+ * would have saved its cost, if it takes no more than a quarter of the free
+ * memory; register-tiled batched otherwise, and where there is no room
+ * for the copy), 1 = plain streaming kernel (B <= 4 per launch,
  * larger B is split into launches; TMA-staged where the row width allows),
  * 2 = batched register-tiled kernel, 3 = plain kernel with register
  * streaming only (the path used for row widths the TMA-staged one skips),
@@ -234,7 +236,9 @@ tpir_status tpir_xor_combine(const void *const *d_srcs, uint32_t count, uint64_t
  * MMA, cta_group::2).  The tensor-core kernel reads a
  * bit-transposed copy of the table (each column's bits over 64 buckets in
  * one word; as large as the table), allocated and built by the first read
- * that uses it and then kept equal to the table by every write and load. */
+ * that uses it and then kept equal to the table by every write and load (a
+ * copy that only batches of the earning kind use: by small writes; a load or a
+ * large batch of writes drops it until they have earned another). */
 tpir_status tpir_db_set_kernel(tpir_db *db, int kernel);
 
 /* Autotuner of the batched read.  For this table and a batch of B requests

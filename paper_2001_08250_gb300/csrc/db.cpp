@@ -138,6 +138,25 @@ uint32_t next_counter_slot() {
   return next.fetch_add(1, std::memory_order_relaxed) % kItemCounterSlots;
 }
 
+// The register-tiled kernel: 10 us and the largest of its operations (17.5 a ps),
+// the table's bytes, a start-up where warps share the buckets, and 0.3 ns a bucket;
+// the tensor-core one: its plan's estimate.  Against 640 measured pairs (rows of 16
+// bytes to 16 KiB, tables of 256 KiB to 1 GiB, 5 .. 1 024 requests) the saving is
+// under-estimated, by a third in the median, but for a few microseconds at tables
+// whose copy costs as little.
+double mid_save(tpir_db* db, uint32_t B) {
+  if (db->save_B == B) return db->save_us;
+  const Shape s = make_job(db, nullptr, B, nullptr).shape;
+  const double n = static_cast<double>(db->n), bytes = n * db->row_bytes;
+  const double tiles = static_cast<double>((B + s.bt() - 1) / s.bt()) * ((db->Wd + s.wt() - 1) / s.wt());
+  double lop3 = std::max(tiles * s.bt() * s.wt() * n / 1.75e7, std::max(1.1 * bytes / 6.8e6, 0.3e-3 * n));
+  if (s.wk >= 4) lop3 = std::max(lop3, std::min(14.0, 0.004 * n));
+  const double tensor = std::max(gf2_tmem_clk(db->n, db->Wd, B, false) / 2020.0, 1.05 * bytes / 6.8e6 + 4.0);
+  db->save_us = 10.0 + lop3 - (tensor + 2.5);
+  db->save_B = B;
+  return db->save_us;
+}
+
 int told_kernel(const tpir_db* db, uint32_t B) {
   if (db->forced_kernel) return db->forced_kernel;
   KernelPlan kp;
@@ -145,26 +164,28 @@ int told_kernel(const tpir_db* db, uint32_t B) {
   return kp.kernel == 5 && db->tt_skip ? 2 : kp.kernel;  // (no room for its copy)
 }
 
-int auto_kernel(const tpir_db* db, uint32_t B) {
+int auto_kernel(tpir_db* db, uint32_t B) {
   if (const int told = told_kernel(db, B)) return told;
   // plain stream for a few requests; the tensor-core kernel for large batches
-  // on wide rows, and for the others it is faster at (tensor_mid) once the
-  // table has its transposed copy, or had one such batch before: the first
-  // runs on the register-tiled kernel, so that a table read once does not pay
-  // for the copy
+  // on wide rows, and for the others it is faster at (tensor_mid) where the table
+  // has its transposed copy or is worth one (copyrule.h)
   if (B <= kPlainMaxB) return 1;
-  if (tensor_mid(db, B))
-    return db->tt_valid || (db->mid_reads && !db->tt_skip && !db->tt_scarce) ? 5 : 2;
+  if (tensor_mid(db, B)) {
+    if (db->tt_valid) return 5;
+    if (db->tt_skip || db->tt_scarce) return 2;
+    const double bytes = static_cast<double>(tcopy_bytes(db->n, db->row_bytes));
+    return db->rule.make(mid_save(db, B), copy_build_us(bytes), db->d_tt ? 0.0 : copy_alloc_us(bytes)) ? 5 : 2;
+  }
   return B >= kTensorMinB && db->Wd >= kTensorMinWd && !db->tt_skip ? 5 : 2;
 }
 
 // Batches other than the large ones on wide rows that the tensor-core kernel
-// reads faster than the register-tiled one (us, tensor / register-tiled: 8 192
-// x 4 KiB 13 / 31 at 8 requests, 17 / 25 at 32; 32 768 x 4 KiB 38 / 32, 38 / 39,
-// 38 / 44, 39 / 70 at 5, 8, 16, 32; 131 072 x 4 KiB 127 / 98, 127 / 144 at 8, 16;
-// 200 003 x 256 bytes 18 / 68 at 5; 200 003 x 128 bytes 14 / 93 at 64): up to 8
-// requests the register-tiled kernel streams large tables of wide rows from
-// HBM at a higher rate.
+// reads faster than the register-tiled one (us, tensor / register-tiled: 8 203
+// x 4 KiB 14 / 35 at 8 requests, 15 / 28 at 32; 32 813 x 4 KiB 35 / 38, 35 / 38,
+// 35 / 47, 36 / 73 at 5, 8, 16, 32; 65 565 x 4 KiB 59 / 59, 59 / 81 and 262 200 x
+// 4 KiB 199 / 189, 200 / 281 at 8, 16; 262 200 x 256 bytes 20 / 91 at 5; 262 200 x
+// 128 bytes 16 / 136 at 64): up to 8 requests the register-tiled kernel streams
+// large tables of wide rows from HBM as fast.
 bool tensor_mid(const tpir_db* db, uint32_t B) {
   if (B <= kPlainMaxB || (B >= kTensorMinB && db->Wd >= kTensorMinWd)) return false;
   if (db->row_bytes > (1u << 27)) return false;  // (the copy's tensor map counts columns in 32 bits)
@@ -181,16 +202,20 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
   const int kernel = kernel_choice ? kernel_choice : auto_kernel(db, B);
   if (kernel_used) *kernel_used = kernel;
   cudaError_t e = cudaSuccess;
-  if (kernel == 5 && (!tensor_mid(db, B) || told_kernel(db, B) == 5)) db->tt_wanted = true;
+  // a batch for which nothing but the rule asks for the copy
+  const bool unasked = kernel_choice == 0 && tensor_mid(db, B) && told_kernel(db, B) == 0;
+  if (kernel == 5 && !unasked) db->tt_wanted = true;
+  const bool by_rule = unasked && !db->tt_wanted;
   if (kernel == 5 && kernel_choice == 0 && db->forced_kernel == 0) {
     // no room for the copy: the register-tiled kernel
+    const bool make = by_rule && !db->tt_valid;
     e = tcopy_ensure(db, st);
     if (e == cudaErrorMemoryAllocation)
       return enqueue_read(db, d_req - db->req_off, B, d_out, st, d_seeds, kernel_used, 2);
     if (e != cudaSuccess) return cuda_status(e);
-  } else if (kernel == 2 && tensor_mid(db, B)) {
-    db->mid_reads = 1;
+    if (make) db->rule.built(copy_build_us(tcopy_bytes(db->n, db->row_bytes)));
   }
+  if (by_rule) db->rule.read(mid_save(db, B));
   if (kernel == 1 || kernel == 3) {
     const uint32_t* T = reinterpret_cast<const uint32_t*>(db->d_table);
     for (uint32_t b0 = 0; b0 < B && e == cudaSuccess; b0 += kPlainMaxB) {
@@ -407,6 +432,7 @@ tpir_status enqueue_multi(const tpir_read_job* jobs, uint32_t njobs, cudaStream_
         continue;
       }
       if (e != cudaSuccess) return cuda_status(e);
+      if (!q.db->tt_wanted) q.db->rule.read(mid_save(q.db, q.B));
       M4Request t = r;
       t.Tt = q.db->d_tt;
       tc.push_back(t);

@@ -99,6 +99,9 @@ cudaError_t launch_tcopy(const tpir_db* db, const void* src, const TcopyBlocks& 
 
 }  // namespace
 
+// Slots (of 64 buckets) up to which writes update a copy that only smaller batches use.
+constexpr size_t kTcopyFewSlots = 16;
+
 uint64_t tcopy_bytes(uint64_t n, uint32_t row_bytes) { return (n + 63) / 64 * 64 * row_bytes; }
 
 cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
@@ -157,17 +160,22 @@ bool tcopy_load(tpir_db* db, const void* src, cudaStream_t st, cudaError_t* e) {
 cudaError_t tcopy_after_load(tpir_db* db, cudaStream_t st) {
   db->tt_skip = 0;
   db->tt_scarce = false;
-  if (!db->d_tt) return cudaSuccess;  // built on first use
+  if (!db->tt_wanted) db->rule.changed(copy_build_us(tcopy_bytes(db->n, db->row_bytes)));
   db->tt_valid = false;
-  if (!db->tt_wanted) {  // only smaller batches used it: made again by the second of them
-    db->mid_reads = 0;
-    return cudaSuccess;
-  }
-  return tcopy_ensure(db, st);
+  // (built on first use; where only smaller batches used it, again when it is worth it)
+  return db->d_tt && db->tt_wanted ? tcopy_ensure(db, st) : cudaSuccess;
 }
 
 cudaError_t tcopy_after_moves(tpir_db* db, const MoveOp* ops, size_t nops, cudaStream_t st) {
-  if (!db->d_tt || !db->tt_valid || nops == 0) return cudaSuccess;
+  if (nops == 0) return cudaSuccess;
+  const double build = copy_build_us(tcopy_bytes(db->n, db->row_bytes));
+  if (!db->tt_valid) {
+    if (nops > kTcopyFewSlots)
+      db->rule.changed(build);
+    else
+      db->rule.wrote(kCopyUpdateUs, build);
+    return cudaSuccess;
+  }
   TcopyBlocks bl{};
   std::vector<uint64_t> kbs;
   kbs.reserve(nops);
@@ -176,9 +184,9 @@ cudaError_t tcopy_after_moves(tpir_db* db, const MoveOp* ops, size_t nops, cudaS
       kbs.push_back(ops[i].dst / db->d / 64 * db->d + ops[i].dst % db->d);
   std::sort(kbs.begin(), kbs.end());
   kbs.erase(std::unique(kbs.begin(), kbs.end()), kbs.end());
-  if (!db->tt_wanted && kbs.size() > 16) {  // as after a load
+  if (!db->tt_wanted && (kbs.size() > kTcopyFewSlots || db->rule.wrote(kCopyUpdateUs, build))) {
+    db->rule.changed(build);  // as after a load
     db->tt_valid = false;
-    db->mid_reads = 0;
     return cudaSuccess;
   }
   uint32_t d = db->d;

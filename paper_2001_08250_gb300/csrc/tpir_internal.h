@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/talekpir.h"
+#include "copyrule.h"
 
 namespace tpir {
 
@@ -398,7 +399,9 @@ struct tpir_db {
                            // for again (0 after a load)
   bool tt_scarce = false;  // refused to a smaller batch, as it would have made memory scarce (a
                            // large one still asks for it); until a load
-  uint32_t mid_reads = 0;  // 1: a batch of tensor_mid size was read without the copy
+  tpir::CopyRule rule;     // whether it is made for batches of tensor_mid size
+  uint32_t save_B = 0;     // mid_save of so many requests, kept
+  double save_us = 0;
 };
 
 namespace tpir {
@@ -426,10 +429,12 @@ tpir_status enqueue_read(tpir_db* db, const uint64_t* d_req, uint32_t B, void* d
 // 0: none.
 int told_kernel(const tpir_db* db, uint32_t B);
 // The kernel it takes.
-int auto_kernel(const tpir_db* db, uint32_t B);
+int auto_kernel(tpir_db* db, uint32_t B);
 // A batch, other than the large ones on wide rows, that the tensor-core kernel
 // reads faster than the register-tiled one.
 bool tensor_mid(const tpir_db* db, uint32_t B);
+// What it saves on such a batch, in microseconds (estimated; 0 or less: nothing).
+double mid_save(tpir_db* db, uint32_t B);
 // order stream `st` after the db's last write, and record a read event
 void order_after_writes(tpir_db* db, cudaStream_t st);
 void note_read(tpir_db* db, cudaStream_t st);

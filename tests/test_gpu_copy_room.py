@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 N, D, Z = 1000, 4, 65536  # 250 MiB; one k-chunk
 ROW = D * Z
-MID, LARGE = 16, 64
+MID, LARGE = 32, 64
 
 
 def fill(torch, leave):
@@ -34,15 +34,23 @@ class Table:
         self.db = talekpir.DB(N, D, Z)
         g = torch.Generator(device="cuda")
         g.manual_seed(210)
-        t = torch.empty(N, ROW // 8, dtype=torch.int64, device="cuda").random_(generator=g)
-        self.db.load_async(t)
+        self.table = torch.empty(N, ROW // 8, dtype=torch.int64, device="cuda").random_(generator=g)
+        self.load()
         self.R = to_dev(synth.random_bits(LARGE, N, seed=211))
         self.out = dev_out(LARGE, ROW)
+        self.expect()
+        torch.cuda.synchronize()
+
+    def load(self):
+        """The same content again."""
+        self.db.load_async(self.table)
+
+    def expect(self):
+        """Replies of the table as it now is, by the register-tiled kernel."""
         self.db.set_kernel(2)
         self.db.read_batch_async(self.R, LARGE, self.out)
         self.expected = self.out.clone()
         self.db.set_kernel(0)
-        torch.cuda.synchronize()
 
     def read(self, B):
         """One read of B requests: its launches (replies checked)."""
@@ -59,7 +67,7 @@ def test_a_refusal_for_small_batches_leaves_large_ones_their_copy():
     t = Table()
     x = fill(torch, 640 << 20)
     try:
-        assert [t.read(MID) for _ in range(4)] == [2] * 4  # refused: over a quarter of 640 MiB
+        assert [t.read(MID) for _ in range(8)] == [2] * 8  # refused: over a quarter of 640 MiB
         assert t.read(LARGE) == 2  # copy and scan
         assert t.read(LARGE) == 1
         assert t.read(MID) == 1
@@ -78,7 +86,7 @@ def test_a_tuned_tensor_kernel_without_room_for_its_copy(tmp_path):
     plan = tmp_path / "plan.json"
     plan.write_text('{"plans": [\n' + "".join(
         '{"row_words": %d, "batch_class": %d, "n_class": 10, "kernel": 5, "tensor_mode": 1, '
-        '"tensor_kc_rows": 0, "tensor_loads": 0}\n' % (ROW // 4, c) for c in (4, 6)) + "]}\n")
+        '"tensor_kc_rows": 0, "tensor_loads": 0}\n' % (ROW // 4, c) for c in (5, 6)) + "]}\n")
     talekpir.tune_load(str(plan))
     x = fill(torch, 160 << 20)
     try:
@@ -108,14 +116,13 @@ def test_a_tuned_small_batch_has_its_copy_as_a_large_one(tmp_path):
     torch = require_cuda()
     t = Table()
     plan = tmp_path / "plan.json"
-    plan.write_text('{"plans": [\n{"row_words": %d, "batch_class": 4, "n_class": 10, "kernel": 5, '
+    plan.write_text('{"plans": [\n{"row_words": %d, "batch_class": 5, "n_class": 10, "kernel": 5, '
                     '"tensor_mode": 1, "tensor_kc_rows": 0, "tensor_loads": 0}\n]}\n' % (ROW // 4))
-    table = torch.as_tensor(t.db.dump()).cuda()
     talekpir.tune_load(str(plan))
     x = fill(torch, 640 << 20)
     try:
         assert [t.read(MID) for _ in range(2)] == [2, 1]  # copy and scan, scan
-        t.db.load_async(table)
+        t.load()
         assert t.read(MID) == 1
     finally:
         talekpir.tune_clear()

@@ -138,18 +138,18 @@ uint32_t next_counter_slot() {
   return next.fetch_add(1, std::memory_order_relaxed) % kItemCounterSlots;
 }
 
-// The register-tiled kernel: 10 us and the largest of its operations (17.5 a ps),
-// the table's bytes, a start-up where warps share the buckets, and 0.3 ns a bucket;
-// the tensor-core one: its plan's estimate.  Against 640 measured pairs (rows of 16
-// bytes to 16 KiB, tables of 256 KiB to 1 GiB, 5 .. 1 024 requests) the saving is
-// under-estimated, by a third in the median, but for a few microseconds at tables
-// whose copy costs as little.
+// The register-tiled kernel: 10 us and the largest of its operations (17.5 a ps, 15
+// in tiles of up to 16 requests), the table's bytes, a start-up where warps share the
+// buckets, and 0.3 ns a bucket; the tensor-core one: its plan's estimate.  Against
+// 640 measured pairs (rows of 16 bytes to 16 KiB, tables of 256 KiB to 1 GiB, 5 ..
+// 1 024 requests) the saving is under-estimated, by a quarter in the median, but for a
+// few microseconds at tables whose copy costs as little.
 double mid_save(tpir_db* db, uint32_t B) {
   if (db->save_B == B) return db->save_us;
   const Shape s = make_job(db, nullptr, B, nullptr).shape;
   const double n = static_cast<double>(db->n), bytes = n * db->row_bytes;
   const double tiles = static_cast<double>((B + s.bt() - 1) / s.bt()) * ((db->Wd + s.wt() - 1) / s.wt());
-  double lop3 = std::max(tiles * s.bt() * s.wt() * n / 1.75e7, std::max(1.1 * bytes / 6.8e6, 0.3e-3 * n));
+  double lop3 = std::max(tiles * s.bt() * s.wt() * n / (s.bt() <= 16 ? 1.5e7 : 1.75e7), std::max(1.1 * bytes / 6.8e6, 0.3e-3 * n));
   if (s.wk >= 4) lop3 = std::max(lop3, std::min(14.0, 0.004 * n));
   const double tensor = std::max(gf2_tmem_clk(db->n, db->Wd, B, false) / 2020.0, 1.05 * bytes / 6.8e6 + 4.0);
   db->save_us = 10.0 + lop3 - (tensor + 2.5);

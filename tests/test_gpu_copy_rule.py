@@ -1,5 +1,5 @@
 """Routes of batches of 32, 47 and 16 requests of a 250 MiB table (estimated savings 61,
-181 and 1.5 us a batch; copy 125 us, its allocation 126), told apart by launches: 2 on
+181 and 12 us a batch; copy 125 us, its allocation 126), told apart by launches: 2 on
 the register-tiled kernel or with the copy's build, 1 with the copy."""
 
 import numpy as np

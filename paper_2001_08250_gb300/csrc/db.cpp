@@ -58,8 +58,31 @@ bool grow_pinned(void** p, uint64_t* cap, uint64_t need) {
   return true;
 }
 
+// The stream's id, which unlike its handle is not given to another stream later;
+// 0: not to be had (the per-thread stream's handle stands for several).
+static unsigned long long stream_id(cudaStream_t st) {
+  unsigned long long id = 0;
+  if (st == cudaStreamPerThread || cudaStreamGetId(st, &id) != cudaSuccess) return 0;
+  return id + 1;
+}
+
+cudaError_t note_write(tpir_db* db, cudaStream_t st) {
+  db->seen_stream = 0;
+  return cudaEventRecord(db->last_write, st);
+}
+
+// A stream that has waited for the last write once is in order from then on.  A
+// wait for each read, where the write is still running, would keep the read's kernels
+// from starting early behind those of the read before (a load and three reads of
+// 8 requests of 32 768 x 4 KiB: 192 us, 162 without).  A captured stream waits each time:
+// the captured wait on work outside fails.
 void order_after_writes(tpir_db* db, cudaStream_t st) {
-  if (db->epoch > 0 || db->last_write) cudaStreamWaitEvent(st, db->last_write, 0);
+  const unsigned long long id = stream_id(st);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool keep = id && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (keep && db->seen_stream == id) return;
+  const cudaError_t e = cudaStreamWaitEvent(st, db->last_write, 0);
+  db->seen_stream = keep && e == cudaSuccess ? id : 0;
 }
 
 void note_read(tpir_db* db, cudaStream_t st) {
@@ -334,7 +357,7 @@ tpir_status apply_writes_core(tpir_db* db, uint32_t count, const uint64_t* b1, c
       if (e == cudaSuccess) e = cudaEventRecord(stg.done, st);
       if (e == cudaSuccess) e = tcopy_after_moves(db, ops.data(), ops.size(), st);
     }
-    if (e == cudaSuccess) e = cudaEventRecord(db->last_write, st);
+    if (e == cudaSuccess) e = note_write(db, st);
     if (e != cudaSuccess) {
       take_back();
       return cuda_status(e);
@@ -379,7 +402,7 @@ tpir_status bloom_insert_core(tpir_db* db, const uint64_t* pos, uint32_t count, 
     i += seg;
   }
   if (e == cudaSuccess) e = cudaEventRecord(stg.done, st);
-  if (e == cudaSuccess) e = cudaEventRecord(db->last_write, st);
+  if (e == cudaSuccess) e = note_write(db, st);
   return cuda_status(e);
 }
 
@@ -570,7 +593,7 @@ tpir_db* tpir_db_create(uint64_t n, uint32_t d, uint32_t msg_bytes) {
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&db->stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&db->last_write, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&db->stream_mark, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventRecord(db->last_write, db->stream);
+  if (e == cudaSuccess) e = note_write(db, db->stream);
   if (e != cudaSuccess) {
     set_error(cuda_status(e));
     tpir_db_destroy(db);
@@ -691,7 +714,7 @@ tpir_status tpir_db_load(tpir_db* db, const void* host_table, size_t bytes) {
   order_writes_after_reads(db, db->stream);
   e = cudaMemcpyAsync(db->d_table, host_table, bytes, cudaMemcpyHostToDevice, db->stream);
   if (e == cudaSuccess) e = tcopy_after_load(db, db->stream);
-  if (e == cudaSuccess) e = cudaEventRecord(db->last_write, db->stream);
+  if (e == cudaSuccess) e = note_write(db, db->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(db->stream);
   if (e != cudaSuccess) return cuda_status(e);
   db->meta->clear();
@@ -708,7 +731,7 @@ tpir_status tpir_db_load_async(tpir_db* db, const void* src, size_t bytes, void*
     e = cudaMemcpyAsync(db->d_table, src, bytes, cudaMemcpyDefault, st);
     if (e == cudaSuccess) e = tcopy_after_load(db, st);
   }
-  if (e == cudaSuccess) e = cudaEventRecord(db->last_write, st);
+  if (e == cudaSuccess) e = note_write(db, st);
   if (e != cudaSuccess) return cuda_status(e);
   db->meta->clear();
   return TPIR_OK;
@@ -929,7 +952,7 @@ tpir_status tpir_read_multi_graph_create(const tpir_read_job* jobs, uint32_t njo
     db->tt_wanted = true;  // replays read the copy as it then is
     if (e == cudaSuccess) e = tcopy_ensure(db, db->stream);
     if (e == cudaErrorMemoryAllocation && db->forced_kernel == 0) continue;  // read by another kernel
-    if (e == cudaSuccess) e = cudaEventRecord(db->last_write, db->stream);
+    if (e == cudaSuccess) e = note_write(db, db->stream);
     if (e != cudaSuccess) {
       delete g;
       return cuda_status(e);
@@ -1058,7 +1081,7 @@ tpir_status tpir_bloom_or_vector(tpir_db* db, const uint64_t* vec) {
   if (e == cudaSuccess)
     e = launch_bloom_or(bl.d_deltas + static_cast<uint64_t>(bl.cur) * bl.words, db->stage.d_pos,
                         bl.m, db->stream);
-  if (e == cudaSuccess) e = cudaEventRecord(db->last_write, db->stream);
+  if (e == cudaSuccess) e = note_write(db, db->stream);
   if (e != cudaSuccess) return cuda_status(e);
   bl.count += 1;
   return TPIR_OK;

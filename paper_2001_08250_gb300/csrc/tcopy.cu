@@ -129,8 +129,9 @@ cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
   TcopyBlocks all{};
   cudaError_t e = launch_tcopy(db, db->d_table, all, st);
   // reads on other streams come after the copy as they come after a write
-  if (e == cudaSuccess) e = cudaEventRecord(db->last_write, st);
+  if (e == cudaSuccess) e = note_write(db, st);
   if (e == cudaSuccess) db->tt_valid = true;
+  if (e == cudaSuccess) order_after_writes(db, st);  // the read that comes next as well
   return e;
 }
 

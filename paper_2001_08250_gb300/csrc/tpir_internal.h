@@ -372,6 +372,7 @@ struct tpir_db {
   int forced_kernel = 0;
   cudaStream_t stream = nullptr;        // the db's own stream (writes, sync reads)
   cudaEvent_t last_write = nullptr;     // recorded after each write
+  unsigned long long seen_stream = 0;   // the stream that waited for it last (0: none)
   cudaEvent_t stream_mark = nullptr;    // marks the db stream for foreign-stream writes
   std::vector<std::pair<cudaStream_t, cudaEvent_t>> read_events;  // async reads per stream
   tpir::CuckooMeta* meta = nullptr;
@@ -437,6 +438,8 @@ bool tensor_mid(const tpir_db* db, uint32_t B);
 double mid_save(tpir_db* db, uint32_t B);
 // order stream `st` after the db's last write, and record a read event
 void order_after_writes(tpir_db* db, cudaStream_t st);
+// records last_write: after each write, on its stream
+cudaError_t note_write(tpir_db* db, cudaStream_t st);
 void note_read(tpir_db* db, cudaStream_t st);
 // A batch of writes: host-side placement, device moves enqueued on `st`
 // using `stg` (which must be free); records db->last_write on `st`.

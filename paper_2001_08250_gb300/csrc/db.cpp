@@ -1137,6 +1137,7 @@ static cudaMemPool_t scratch_pool() {
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
     cudaMemPool_t p = nullptr;
+    const RelaxedCapture relaxed;
     if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;

@@ -230,6 +230,15 @@ struct TcopyBlocks {
 };
 static_assert(sizeof(TcopyBlocks) + 64 < 32000, "kernel parameters must stay below 32 KB");
 uint64_t tcopy_bytes(uint64_t n, uint32_t row_bytes);
+// Allocations in calls that may come while this thread captures a stream: without
+// it they would end the capture (what they allocate is no part of it).
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  RelaxedCapture(const RelaxedCapture&) = delete;
+  RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+};
 int read_device_status_and_clear(int* status);
 // Device address of the status word on the current device (for kernels in
 // other translation units).

@@ -108,6 +108,7 @@ cudaError_t tcopy_ensure(tpir_db* db, cudaStream_t st) {
   if (db->tt_valid) return cudaSuccess;
   if (!db->d_tt) {
     const uint64_t bytes = tcopy_bytes(db->n, db->row_bytes);
+    const RelaxedCapture relaxed;  // (a read on another stream than the captured one)
     if (!db->tt_wanted) {  // only for the smaller batches: not if it would make memory scarce
       size_t free_b = 0, total_b = 0;
       if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || bytes > free_b / 4) {

@@ -248,7 +248,7 @@ tpir_status tpir_db_set_kernel(tpir_db *db, int kernel);
  *     width and the row tile width, and the rows per pipeline stage);
  *   - the tensor-core kernel's schedules (the table operand in tensor memory;
  *     above 128 requests also items on CTA pairs; each with k-chunks of the
- *     planned size and of 2048 .. 32768 buckets);
+ *     planned size and of those sizes from 2048 to 32768 buckets that it holds);
  *   - the Four-Russians kernel (B >= 32, rows of 256 bytes or more) and the
  *     plain kernel (B <= 16);
  * and keeps (a) the fastest tile shape for every later launch of the
@@ -269,7 +269,7 @@ typedef struct {
     uint32_t tensor_mode;      /* its tensor-core schedule: 1 table operand in tensor memory, 2
                                   items on CTA pairs (above 128 requests) */
     uint32_t tensor_kc_rows;   /* k-chunk buckets (0: planned size) */
-    uint32_t tensor_loads;     /* 1: request words loaded by threads, not TMA */
+    uint32_t tensor_loads;     /* 0 (saved plans may hold 1, an earlier schedule: read as mode 1) */
     uint32_t tensor_candidates;
     double us_lop3, us_tensor, us_m4rm, us_plain;  /* best of each kernel (0: not timed) */
 } tpir_tune_result;
@@ -284,8 +284,8 @@ tpir_status tpir_tune_clear(void);
  * workload): job i reads B_i rows of d_req_bits_i against db_i into d_out_i.
  * Tables may differ in n, d and msg_bytes.  Jobs of >= 48 requests on rows of
  * >= 256 bytes, and smaller ones the tensor-core kernel is faster at on tables
- * that have its copy, share one launch of the tensor-core kernel (per 64 jobs),
- * the others one launch of the register-tiled kernel (a db forced to kernel 4 sends its jobs
+ * that have its copy, share one launch of the tensor-core kernel per block layout
+ * (up to 112 requests, above) and 64 jobs, the others one launch of the register-tiled kernel (a db forced to kernel 4 sends its jobs
  * to the Four-Russians kernel instead: one launch for jobs of up to 256
  * requests, one for larger ones; forced to 2, to the register-tiled one).  A
  * job with d_seeds (B x 32 bytes, 16-byte aligned) is masked as in

@@ -769,13 +769,14 @@ uint32_t t_min_chunks(const TJob& j) {
 }
 
 // k-chunks and column splits of a one-job launch: the least rounds x item
-// time over the chunk counts from the fewest that fit on.  Returns the clocks.
-double t_plan(TJob& j, uint32_t grid) {
+// time over the chunk counts from the fewest that fit on, or with chunks of
+// `fixed` words (0: none given).  Returns the clocks.
+double t_plan(TJob& j, uint32_t grid, uint32_t fixed = 0) {
   const uint32_t c0 = t_min_chunks(j);
   double best = 1e300;
   uint32_t bw = 1, bs = 1;
   for (uint32_t c = c0; c <= std::min<uint32_t>(j.nw, c0 + 40); ++c) {
-    const uint32_t kw = (j.nw + c - 1) / c;
+    const uint32_t kw = fixed ? fixed : (j.nw + c - 1) / c;
     const uint64_t per = static_cast<uint64_t>(j.mbs) * ((j.nw + kw - 1) / kw);
     for (uint32_t k = 1; k <= 4; ++k) {
       uint32_t s = static_cast<uint32_t>(std::min<uint64_t>(j.tiles, k * grid / per));
@@ -792,6 +793,7 @@ double t_plan(TJob& j, uint32_t grid) {
         bs = s;
       }
     }
+    if (fixed) break;
   }
   t_set_chunks(j, bw, bs);
   return best;
@@ -835,6 +837,10 @@ double gf2_tmem_clk(uint64_t n, uint32_t Wd, uint32_t B, bool masked) {
   return 1.04 * (clk + (masked && j.kcs == 1 ? 4000.0 : 1000.0));
 }
 
+uint32_t gf2_tmem_max_rows(uint32_t B) {
+  return 64u * t_max_words(t_job(nullptr, 0, B, nullptr, nullptr, 64, 4).mb_rows);
+}
+
 cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const uint64_t* R,
                             uint32_t words64, uint32_t B, uint32_t* out, const uint8_t* seeds,
                             cudaStream_t st, uint32_t kc_rows) {
@@ -843,8 +849,7 @@ cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const u
   L.njobs = 1;
   TJob J = t_job(R, words64, B, out, seeds, n, Wd);
   const uint32_t grid = static_cast<uint32_t>(device_sm_count());
-  t_plan(J, grid);
-  if (kc_rows) t_set_chunks(J, std::min(t_max_words(J.mb_rows), std::max<uint32_t>(1, kc_rows / 64)), J.splits);
+  t_plan(J, grid, kc_rows ? std::min(t_max_words(J.mb_rows), std::max<uint32_t>(1, kc_rows / 64)) : 0u);
   const uint64_t items = static_cast<uint64_t>(J.mbs) * J.kcs * J.splits;
   if (items > 0xFFFFFFFFull) return cudaErrorInvalidValue;
   L.total_items = static_cast<uint32_t>(items);

@@ -187,11 +187,12 @@ tpir_status tpir_autotune(tpir_db* db, uint32_t B, uint32_t reps, tpir_tune_resu
   if (e == cudaSuccess && tcopy_ensure(db, st) == cudaSuccess) {  // (no room for the copy: not tried)
     std::vector<GSched> scheds;
     // mode 1 (table operand in tensor memory) and, above 128 requests, mode 2
-    // (CTA pairs), each with planned and with given k-chunks
+    // (CTA pairs), each with planned k-chunks and with given ones that it holds
     for (uint32_t mode = 1; mode <= (B > 128 ? 2u : 1u); ++mode) {
       scheds.push_back(GSched{mode, 0, 0});
       for (uint32_t kc : {2048u, 4096u, 8192u, 16384u, 32768u})
-        if (kc < (db->n + 255) / 256 * 256) scheds.push_back(GSched{mode, kc, 0});
+        if (kc < (db->n + 255) / 256 * 256 && (mode == 2 || kc <= gf2_tmem_max_rows(B)))
+          scheds.push_back(GSched{mode, kc, 0});
     }
     for (const GSched& sc : scheds) {
       const double us = time_it([&]() {

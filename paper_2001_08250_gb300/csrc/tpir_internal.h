@@ -166,6 +166,8 @@ cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const u
                             uint32_t words64, uint32_t B, uint32_t* out, const uint8_t* seeds,
                             cudaStream_t st, uint32_t kc_rows = 0);
 cudaError_t launch_gf2_tmem_multi(const M4Request* reqs, uint32_t count, cudaStream_t st);
+// The most buckets of a k-chunk for batches of B requests.
+uint32_t gf2_tmem_max_rows(uint32_t B);
 // Its estimated clocks on the whole device, launch included.
 double gf2_tmem_clk(uint64_t n, uint32_t Wd, uint32_t B, bool masked);
 int device_sm_count();

@@ -115,3 +115,39 @@ def test_items_of_one_tile_one_after_another(n, d, z, B):
             talekpir.read_multi_async([(db, B, dR, out), (db2, B2, dR2, out2)])
         assert np.array_equal(to_host(out), exp) and np.array_equal(to_host(out2), exp2)
     assert talekpir.device_status() == talekpir.OK
+
+
+@pytest.mark.parametrize("n,B,count", [(32768, 128, 2), (32768, 112, 2), (32768, 16, 5), (32768, 256, 7), (2048, 64, 1),
+                                       (100000, 16, 5), (100000, 8, 5)])
+def test_autotune_times_each_schedule_once(n, B, count):
+    """The tensor-memory form's k-chunks hold 2 816 buckets at 128 requests a block,
+    3 072 at 112, 21 504 at 16: sizes that it would cut to those are not candidates
+    (CTA pairs, above 128 requests, hold all)."""
+    require_cuda()
+    with talekpir.DB(n, 1, 2048) as db:
+        try:
+            r = db.autotune(B, 1)
+            assert r["tensor_candidates"] == count
+        finally:
+            talekpir.tune_clear()
+
+
+@pytest.mark.parametrize("kc", [256, 2048, 16384, 32768])
+@pytest.mark.parametrize("B", [16, 100, 128, 200])
+def test_given_chunks_bit_exact(kc, B, tmp_path):
+    """Plans with k-chunks of a given size, also of one that the form cuts."""
+    require_cuda()
+    n, d, z = 9000, 2, 80
+    T = synth.table_bytes(n, d, z, seed=185, table=n)
+    R = synth.random_bits(B, n, seed=186, table=n)
+    plan = tmp_path / "plan.json"
+    plan.write_text('{"plans": [\n{"row_words": %d, "batch_class": %d, "n_class": 14, "kernel": 5, "tensor_mode": 1, '
+                    '"tensor_kc_rows": %d, "tensor_loads": 0}\n]}\n' % (d * z // 4, (B - 1).bit_length(), kc))
+    talekpir.tune_load(str(plan))
+    try:
+        with talekpir.DB(n, d, z) as db:
+            db.load(T)
+            assert np.array_equal(db.read_batch(R), oracle.read_batch(T, n, d, z, R))
+    finally:
+        talekpir.tune_clear()
+    assert talekpir.device_status() == talekpir.OK

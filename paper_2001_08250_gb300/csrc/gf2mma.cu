@@ -798,7 +798,8 @@ cudaError_t g_launch_pair(const uint64_t* Tt, uint64_t n, uint32_t Wd, const uin
   L.total_items = static_cast<uint32_t>(items);
   cudaError_t e = gf2_table_map(Tt, n, Wd, kPCols, &L.map);
   if (e != cudaSuccess) return e;
-  if (J.split == 1) e = launch_init_replies(reinterpret_cast<uint4*>(out), B, Wd / 4, seeds, st);
+  // (masks in CTAs of 64 threads, some of which fit beside a CTA of the scan before)
+  if (J.split == 1) e = launch_init_replies(reinterpret_cast<uint4*>(out), B, Wd / 4, seeds, st, 64);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(2 * std::min<uint64_t>(items, pairs)));

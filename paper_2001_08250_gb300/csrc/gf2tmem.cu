@@ -799,12 +799,25 @@ double t_plan(TJob& j, uint32_t grid, uint32_t fixed = 0) {
   return best;
 }
 
-// The replies that a launch XOR-reduces into, initialised before it.
+// The replies that a launch XOR-reduces into, initialised before it.  Masks take
+// time: they are spread over the SMs in CTAs of 64 threads, one of which fits beside a
+// CTA of the scan before it (G = 1).  Beside one of G = 2, which leaves no registers,
+// none does: started early, they go to the first SMs that it leaves, four at most to
+// each by the shared memory they ask for (48 masked reads of 32 768 x 4 KiB 37 us, 45
+// in CTAs of 256 without, 39 when they wait for the scan's end).
 template <int NJ>
-cudaError_t t_init(const TLaunch<NJ>& L, cudaStream_t st) {
+cudaError_t t_init(const TLaunch<NJ>& L, int G, cudaStream_t st) {
   bool any = false;
-  for (uint32_t i = 0; i < L.njobs; ++i) any |= L.jobs[i].split == 1;
-  return any ? launch_pdl(gf2_tmem_init_kernel<NJ>, dim3(64, L.njobs), dim3(256), 0, st, L) : cudaSuccess;
+  uint64_t blocks = 0;  // keystream blocks of the job with the most masks
+  for (uint32_t i = 0; i < L.njobs; ++i) {
+    if (L.jobs[i].split != 1) continue;
+    any = true;
+    if (L.jobs[i].seeds) blocks = std::max(blocks, static_cast<uint64_t>(L.jobs[i].B) * ((L.jobs[i].Wd + 15) / 16));
+  }
+  if (!any) return cudaSuccess;
+  if (!blocks) return launch_pdl(gf2_tmem_init_kernel<NJ>, dim3(64, L.njobs), dim3(256), 0, st, L);
+  const uint32_t ctas = static_cast<uint32_t>(std::min<uint64_t>((blocks + 63) / 64, 256));
+  return launch_pdl(gf2_tmem_init_kernel<NJ>, dim3(ctas, L.njobs), dim3(64), G == 2 ? 48u * 1024u : 0u, st, L);
 }
 
 template <int NJ, int G>
@@ -856,7 +869,7 @@ cudaError_t launch_gf2_tmem(const uint64_t* Tt, uint64_t n, uint32_t Wd, const u
   L.jobs[0] = J;
   cudaError_t e = gf2_table_map(Tt, n, Wd, kTCols, &L.maps[0]);
   if (e != cudaSuccess) return e;
-  e = t_init(L, st);
+  e = t_init(L, t_groups(J.mb_rows), st);
   if (e != cudaSuccess) return e;
   return t_groups(J.mb_rows) == 2 ? t_scan<1, 2>(L, st) : t_scan<1, 1>(L, st);
 }
@@ -930,8 +943,8 @@ cudaError_t launch_gf2_tmem_multi(const M4Request* reqs, uint32_t count, cudaStr
           part[g].data() + i, static_cast<uint32_t>(std::min<size_t>(kTMultiJobs, part[g].size() - i)), ls.back());
       if (e != cudaSuccess) return e;
     }
-  for (const auto& l : ls) {
-    const cudaError_t e = t_init(l, st);
+  for (size_t i = 0; i < ls.size(); ++i) {
+    const cudaError_t e = t_init(ls[i], layout[i], st);
     if (e != cudaSuccess) return e;
   }
   for (size_t i = 0; i < ls.size(); ++i) {

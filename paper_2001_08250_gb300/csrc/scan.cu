@@ -921,14 +921,15 @@ static bool plain_tma_ok(uint32_t U, int nb) {
 }
 
 cudaError_t launch_init_replies(uint4* out, uint32_t B, uint32_t row_u4, const uint8_t* seeds,
-                                cudaStream_t st) {
+                                cudaStream_t st, uint32_t mask_threads) {
   // one thread per 16-byte word (zeros) or per 64-byte keystream block (masks)
   const uint64_t work = seeds ? static_cast<uint64_t>(B) * ((row_u4 + 3) / 4)
                               : static_cast<uint64_t>(B) * row_u4;
   if (work == 0) return cudaSuccess;
+  const uint32_t threads = seeds ? mask_threads : 256;
   return launch_pdl(init_replies_kernel,
-                    dim3(static_cast<uint32_t>(std::min<uint64_t>((work + 255) / 256, 1024))),
-                    dim3(256), 0, st, out, B, row_u4, seeds);
+                    dim3(static_cast<uint32_t>(std::min<uint64_t>((work + threads - 1) / threads, 1024))),
+                    dim3(threads), 0, st, out, B, row_u4, seeds);
 }
 
 cudaError_t launch_plain(const uint32_t* T, uint64_t n, uint32_t Wd, const uint64_t* R,

@@ -149,7 +149,7 @@ cudaError_t launch_zero_outputs(const ScanLaunch& L, cudaStream_t st);
 // Initialises B replies of row_u4 16-byte words before a scan XOR-reduces into
 // them: zeros, or the masks of `seeds` (PDL-chained).
 cudaError_t launch_init_replies(uint4* out, uint32_t B, uint32_t row_u4, const uint8_t* seeds,
-                                cudaStream_t st);
+                                cudaStream_t st, uint32_t mask_threads = 256);
 // Tensor-core batched read (gf2tmem.cu; gf2mma.cu: the CTA-pair form and the
 // choice between them): the GF(2) product as an exact integer
 // product of 0/1 matrices on tcgen05 (packed e2m1 operands), reduced mod 2.

@@ -203,3 +203,27 @@ def test_masked_read_argument_errors():
         assert L.tpir_mask_generate(S.data_ptr(), 1, 40, O.data_ptr(), None) == talekpir.EINVAL
         assert L.tpir_xor_combine(None, 0, 16, O.data_ptr(), None) == talekpir.EINVAL
     assert talekpir.device_status() == talekpir.OK
+
+
+@pytest.mark.parametrize("n,d,z,B", [(300, 4, 1024, 48), (300, 4, 1024, 112), (300, 4, 1024, 128), (2500, 1, 1024, 100),
+                                     (2500, 4, 1024, 80), (1500, 1, 2048, 384), (5000, 4, 2048, 17), (20011, 3, 368, 250),
+                                     (700, 1, 16, 1000), (9000, 64, 256, 130)])
+def test_masked_replies_where_masks_are_written_or_formed(n, d, z, B):
+    """Masked tensor-core reads whose masks are formed at the stores of one tile a CTA or
+    two, or written before the scan in few CTAs or many, of both block layouts and of CTA
+    pairs; repeated into one buffer, so that each read's masks come behind a scan."""
+    require_cuda()
+    T = synth.table_bytes(n, d, z, seed=190, table=n)
+    R = synth.random_bits(B, n, seed=191, table=n)
+    S = synth.mask_seeds(B, seed=192, table=n)
+    exp = oracle.read_batch_masked(T, n, d, z, R, S)
+    with talekpir.DB(n, d, z) as db:
+        db.load(T)
+        db.set_kernel(5)
+        dR, dS, out = to_dev(R), to_dev(S), dev_out(B, d * z)
+        for _ in range(20):
+            db.read_batch_masked_async(dR, B, dS, out)
+        assert np.array_equal(to_host(out), exp)
+        talekpir.read_multi_async([(db, B, dR, out, dS)])
+        assert np.array_equal(to_host(out), exp)
+    assert talekpir.device_status() == talekpir.OK

@@ -834,7 +834,15 @@ cudaError_t launch_gf2_mma(const uint64_t* Tt, uint64_t n, uint32_t Wd, const ui
   if (rm) {
     const int pairs = rm == 1 ? p_max_pairs<1>() : p_max_pairs<2>();
     uint32_t rows = 0;
-    if (pairs > 0 && (mode == 2 || g_pair_plan(n, Wd, B, pairs, &rows) < gf2_tmem_clk(n, Wd, B, seeds != nullptr)))
+    bool pair = pairs > 0 && mode == 2;
+    if (pairs > 0 && mode == 0) {
+      // (masks formed where a single k-chunk's replies are stored take 1.4 to 7 us; written
+      // before the scan as much more than zeros as in the other form)
+      double clk = g_pair_plan(n, Wd, B, pairs, &rows);
+      if (seeds) clk += rows >= n ? 7000.0 : 2000.0;
+      pair = clk < gf2_tmem_clk(n, Wd, B, seeds != nullptr);
+    }
+    if (pair)
       return rm == 1 ? g_launch_pair<1>(Tt, n, Wd, R, words64, B, out, seeds, st, sched)
                      : g_launch_pair<2>(Tt, n, Wd, R, words64, B, out, seeds, st, sched);
   }

@@ -751,22 +751,41 @@ TJob t_job(const uint64_t* R, uint32_t words64, uint32_t B, uint32_t* out, const
 
 uint32_t t_max_words(uint32_t N) { return (t_groups(N) == 2 ? TLayout<2>::kRes : TLayout<1>::kRes) / (32 * N); }
 
+// How a job's replies are stored with kcs k-chunks (TJob::split).  A masked read of
+// a table so small that every CTA has a tile at most forms the masks where it stores
+// (a keystream block per eight bytes, but no launch before it: 90 masked reads of 1 132
+// x 256 bytes 5.0 us, 6.8 with one); larger ones have them written first, a block
+// per 64 bytes.
+uint32_t t_split(const TJob& j, uint32_t kcs) {
+  if (kcs > 1) return 1;
+  if (!j.seeds) return 0;
+  return static_cast<uint64_t>(j.mbs) * j.tiles <= static_cast<uint64_t>(device_sm_count()) ? 2 : 1;
+}
+// What that adds to a launch, in clocks: the replies' initialisation, or masks
+// formed at the stores of `nt` tiles of an item.
+double t_split_clk(const TJob& j, uint32_t kcs, uint32_t nt) {
+  const uint32_t split = t_split(j, kcs);
+  if (split == 0) return 0.0;
+  if (split == 2) return 1800.0 * nt;
+  return j.seeds && kcs > 1 ? 5000.0 : 3000.0;
+}
+
 void t_set_chunks(TJob& j, uint32_t kc_words, uint32_t splits) {
   j.kc_words = kc_words;
   j.kcs = (j.nw + kc_words - 1) / kc_words;
   j.splits = splits;
-  // a masked read of a table so small that every CTA has a tile at most forms
-  // the masks where it stores (a keystream block per eight bytes, but no launch
-  // before it: 90 masked reads of 1 132 x 256 bytes 5.4 us, 6.8 with one); larger
-  // ones have them written first, a block per 64 bytes
-  const bool small = static_cast<uint64_t>(j.mbs) * j.tiles <= static_cast<uint64_t>(device_sm_count());
-  j.split = j.kcs > 1 ? 1u : !j.seeds ? 0u : small ? 2u : 1u;
+  j.split = t_split(j, j.kcs);
 }
 
 uint32_t t_min_chunks(const TJob& j) {
   const uint32_t maxw = t_max_words(j.mb_rows);
   return (j.nw + maxw - 1) / maxw;
 }
+
+// A launch of however little work: its words have to come, be expanded, multiplied
+// and read back (2 500 x 256 bytes at 48 requests 5.5 us in one k-chunk, 7.2 with ten
+// and their replies' initialisation, which the items' times alone made 4.9).
+constexpr double kTLeastClk = 12500.0;
 
 // k-chunks and column splits of a one-job launch: the least rounds x item
 // time over the chunk counts from the fewest that fit on, or with chunks of
@@ -784,9 +803,8 @@ double t_plan(TJob& j, uint32_t grid, uint32_t fixed = 0) {
       const uint32_t st = (j.tiles + s - 1) / s;
       const uint64_t items = per * s;
       const uint64_t rounds = (items + grid - 1) / grid;
-      // (the replies' initialisation, a launch, costs a read of several k-chunks
-      // 3 000 clocks: a small table is read in one)
-      const double cost = static_cast<double>(rounds) * t_item_clk(j.mb_rows, kw, st) + (kw < j.nw ? 3000.0 : 0.0);
+      const double cost = std::max(static_cast<double>(rounds) * t_item_clk(j.mb_rows, kw, st), kTLeastClk) +
+                          t_split_clk(j, (j.nw + kw - 1) / kw, st);
       if (cost < best) {
         best = cost;
         bw = kw;
@@ -842,12 +860,12 @@ cudaError_t t_scan(TLaunch<NJ>& L, cudaStream_t st) {
 
 }  // namespace
 
-// (with a launch, and the replies' initialisation where there is one; 4 % more
-// than fitted: where the two forms are as close as that, the other one is taken)
+// (with a launch; 4 % more than fitted: where the two forms are as close as that, the other one is taken)
 double gf2_tmem_clk(uint64_t n, uint32_t Wd, uint32_t B, bool masked) {
-  TJob j = t_job(nullptr, 0, B, nullptr, nullptr, n, Wd);
+  static const uint8_t some = 0;  // (a masked job plans as one; nothing is read)
+  TJob j = t_job(nullptr, 0, B, nullptr, masked ? &some : nullptr, n, Wd);
   const double clk = t_plan(j, static_cast<uint32_t>(device_sm_count()));
-  return 1.04 * (clk + (masked && j.kcs == 1 ? 4000.0 : 1000.0));
+  return 1.04 * (clk + 1000.0);
 }
 
 uint32_t gf2_tmem_max_rows(uint32_t B) {

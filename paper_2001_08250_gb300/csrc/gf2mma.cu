@@ -836,10 +836,9 @@ cudaError_t launch_gf2_mma(const uint64_t* Tt, uint64_t n, uint32_t Wd, const ui
     uint32_t rows = 0;
     bool pair = pairs > 0 && mode == 2;
     if (pairs > 0 && mode == 0) {
-      // (masks formed where a single k-chunk's replies are stored take 1.4 to 7 us; written
-      // before the scan as much more than zeros as in the other form)
-      double clk = g_pair_plan(n, Wd, B, pairs, &rows);
-      if (seeds) clk += rows >= n ? 7000.0 : 2000.0;
+      // (masks take 1.4 to 7 us, formed where a single k-chunk's replies are stored or
+      // written before the scan)
+      const double clk = g_pair_plan(n, Wd, B, pairs, &rows) + (seeds ? 7000.0 : 0.0);
       pair = clk < gf2_tmem_clk(n, Wd, B, seeds != nullptr);
     }
     if (pair)

@@ -875,12 +875,13 @@ cudaError_t t_scan(TLaunch<NJ>& L, cudaStream_t st) {
 
 }  // namespace
 
-// (with a launch; 4 % more than fitted: where the two forms are as close as that, the other one is taken)
+// (with a launch and, where masks are reduced into, their share of it that no chunking
+// changes; 4 % more than fitted: where the two forms are as close as that, the other one is taken)
 double gf2_tmem_clk(uint64_t n, uint32_t Wd, uint32_t B, bool masked) {
   static const uint8_t some = 0;  // (a masked job plans as one; nothing is read)
   TJob j = t_job(nullptr, 0, B, nullptr, masked ? &some : nullptr, n, Wd);
   const double clk = t_plan(j, static_cast<uint32_t>(device_sm_count()));
-  return 1.04 * (clk + 1000.0);
+  return 1.04 * (clk + (masked && j.kcs > 1 ? 6000.0 : 1000.0));
 }
 
 uint32_t gf2_tmem_max_rows(uint32_t B) {

@@ -75,7 +75,6 @@ struct GJob {
   uint64_t n;
   uint32_t Wd, words64, B;
   uint32_t n_strips, n_mb, kc_rows;
-  uint32_t item_begin;   // index of this job's first item in the launch
   uint32_t split;        // 0: replies stored; 1: initialised first (zeros or masks)
                          // and XOR-reduced into; 2: masked, stored by their single
                          // writer (one k-chunk, items) with the mask XORed in
@@ -783,7 +782,6 @@ cudaError_t g_launch_pair(const uint64_t* Tt, uint64_t n, uint32_t Wd, const uin
   const uint64_t items = nps * J.n_mb * kcs;
   if (items > 0xFFFFFFFFull) return cudaErrorInvalidValue;
   J.split = kcs > 1 ? 1u : seeds ? 2u : 0u;
-  J.item_begin = 0;
   const uint64_t nw = (n + 63) / 64;
   if (RM == 1) {
     if (g_req_map(R, nw, B, words64, kGStageWords, 128, &L.rmap) != cudaSuccess)

@@ -613,6 +613,9 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
       const TJob& J = L.jobs[it.job];
       const uint32_t N = J.mb_rows, c0 = N > 64 ? 64 * half : 32 * half;
       const bool two = N > 64 && c0 + 32 < N;  // this warp reads a second 32 columns
+      // the next item's requests are announced once both issuers have seen this
+      // item's (asked here, while its first counts are still to come)
+      const bool seen = lane != 0 || !more || mb::wait(&reqe, r & 1u, abort_flag, status, kTWaitNs);
       uint32_t t = it.t0;
       for (uint32_t i = 0; i < it.nt; ++i, t += J.splits, ++te) {
         const uint32_t g = i % kTStreams, c = g ? tc1++ : tc0++, buf = nb2 & c;
@@ -654,11 +657,10 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
         if (more && i + 1 == it.nt) {
           // every tile's MMAs have read the item's requests: the next item's
           // go in before this tile's replies, so that its MMAs start the sooner
-          // (and are announced once both issuers have seen this item's)
           t_load_requests(L.jobs[nx.job], nx, res0, warp - kTEpiWarp0, lane);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
-          if (lane == 0 && mb::wait(&reqe, r & 1u, abort_flag, status, kTWaitNs)) mb::arrive(&reqf);
+          if (lane == 0 && seen) mb::arrive(&reqf);
         }
         const WarpTranspose transpose;  // formed anew for each tile: its registers are the counts' before
         const uint32_t ob = out0 + (te & 1u) * kTOutBytes, oq = ob + (c0 + lane) * 16u + quarter * 4u;

@@ -53,6 +53,8 @@ TRAFFIC_BATCHED_B256 = (136.659968e6 + 3.284480e6 + 136.435200e6 + 0.130304e6 + 
 TRAFFIC_PLAIN_B1 = 134.240768e6 + 3.548928e6
 TRAFFIC_M4RM_B256 = (136.340736e6 + 3.074048e6 + 136.585216e6 + 0.072192e6 + 136.370944e6
                      + 0.116480e6) / 3
+TRAFFIC_GF2TMEM_B256 = (136.396544e6 + 3.328768e6 + 136.418816e6 + 3.598080e6 + 136.406016e6
+                        + 3.475968e6) / 3
 TRAFFIC_GF2MMA_B256 = (135.351040e6 + 2.960640e6 + 135.359488e6 + 0.532736e6 + 135.379200e6
                        + 0.106752e6) / 3
 
@@ -553,7 +555,7 @@ def main() -> None:
             "clocks": ck,
             "roofline": {"bound": "tensor", "achieved": tc_tflops, "peak": tc_peak,
                          "unit": "TFLOP/s", "frac": tc_tflops / tc_peak,
-                         "traffic": None if tmem_head else TRAFFIC_GF2MMA_B256,  # captured for the pair form
+                         "traffic": TRAFFIC_GF2TMEM_B256 if tmem_head else TRAFFIC_GF2MMA_B256,
                          "kernel": ("gf2_tmem_kernel (tcgen05 kind::mxf4, e2m1 0/1 operands, table operand in tensor memory)"
                                     if tmem_head else
                                     "gf2_mma_pair_kernel (tcgen05 cta_group::2 kind::mxf4, e2m1 0/1 operands)"),

@@ -49,11 +49,11 @@
 //
 // Measured (us a launch; before: both operands in shared memory, one CTA an
 // SM): 32 768 x 4 KiB: 33 at 32 requests (68 on the register-tiled kernel), 36
-// at 64 (77), 42 at 112, 45 at 128 (77); 50 021 x 4 160 bytes masked: 66 at 100
-// requests (134); 200 003 x 128 bytes: 12 at 64 (93 on the register-tiled
+// at 64 (77), 42 at 112, 44 at 128 (77); 50 021 x 4 160 bytes masked: 65 at 100
+// requests (134); 200 003 x 128 bytes: 12.5 at 64 (93 on the register-tiled
 // kernel).  Blocks of up to 112 requests with one expander group: 39, 40, 44 and
 // 80, 12.4.  What bounds it: instruction latency and the ALU pipe in the
-// expanders and the issuers (issue slots 55 % used, ALU pipe 53 %, tensor pipe 53 %
+// expanders and the issuers (issue slots 57 % used, ALU pipe 54 %, tensor pipe 56 %
 // at 128 requests; HBM 60 % at 32).
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -724,7 +724,7 @@ __global__ void gf2_tmem_init_kernel(const __grid_constant__ TLaunch<NJ> L) {
 // Blocks of up to 112 requests take the layout with two expander groups.
 int t_groups(uint32_t N) { return N <= TLayout<2>::kAcc ? 2 : 1; }
 // Clocks of an item: W words (K = 64 steps, whole stages of four) of nt tiles at
-// N requests, fitted to the measured launches (24 shapes, within 5 %).  The two
+// N requests, fitted to measured launches.  The two
 // streams together run a step in 0.54 N clocks (the MMA) or 48 (instruction
 // latency); one alone in 115, and it stands still while a tile's counts are read.
 double t_item_clk(uint32_t N, uint32_t W, uint32_t nt) {

@@ -147,7 +147,8 @@ cudaError_t launch_plain(const uint32_t* T, uint64_t n, uint32_t Wd, const uint6
                          cudaStream_t st, int ctas);
 cudaError_t launch_zero_outputs(const ScanLaunch& L, cudaStream_t st);
 // Initialises B replies of row_u4 16-byte words before a scan XOR-reduces into
-// them: zeros, or the masks of `seeds` (PDL-chained).
+// them: zeros, or the masks of `seeds` (PDL-chained; in CTAs of mask_threads, few
+// where a CTA has to fit beside those of the kernel before it).
 cudaError_t launch_init_replies(uint4* out, uint32_t B, uint32_t row_u4, const uint8_t* seeds,
                                 cudaStream_t st, uint32_t mask_threads = 256);
 // Tensor-core batched read (gf2tmem.cu; gf2mma.cu: the CTA-pair form and the

@@ -614,8 +614,10 @@ __global__ void __launch_bounds__(TLayout<G>::kThreads, 1)
       const uint32_t N = J.mb_rows, c0 = N > 64 ? 64 * half : 32 * half;
       const bool two = N > 64 && c0 + 32 < N;  // this warp reads a second 32 columns
       // the next item's requests are announced once both issuers have seen this
-      // item's (asked here, while its first counts are still to come)
-      const bool seen = lane != 0 || !more || mb::wait(&reqe, r & 1u, abort_flag, status, kTWaitNs);
+      // item's (asked by one of the warps whose arrivals announce them, and here, while
+      // the first counts are still to come)
+      const bool seen = warp != kTEpiWarp0 || lane != 0 || !more ||
+                        mb::wait(&reqe, r & 1u, abort_flag, status, kTWaitNs);
       uint32_t t = it.t0;
       for (uint32_t i = 0; i < it.nt; ++i, t += J.splits, ++te) {
         const uint32_t g = i % kTStreams, c = g ? tc1++ : tc0++, buf = nb2 & c;
